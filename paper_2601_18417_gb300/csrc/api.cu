@@ -196,10 +196,9 @@ static void free_built(hofv_ctx* c) {
 // rewrite the face and cell coefficient arrays as double-float pairs
 // (to_df = 1) or back to doubles (0), in place
 static int coef_format(hofv_ctx* c, int to_df) {
-  const int64_t nfco = std::max<int64_t>(c->nftile, 1) * c->S * kTile * c->Q * c->dim;
-  const int64_t ncex = c->nctile * c->S * kTile * c->nlf;
-  launch_coef_format(c->d_fco, nfco, to_df, c->stream);
-  launch_coef_format(c->d_cex, ncex, to_df, c->stream);
+  launch_coef_format(c->d_fco, std::max<int64_t>(c->nftile, 1) * c->S, kTile * c->Q, c->dim, to_df,
+                     c->stream);
+  launch_coef_format(c->d_cex, c->nctile * c->S, kTile, c->nlf, to_df, c->stream);
   c->prec = to_df ? HOFV_PREC_DF64 : HOFV_PREC_FP64;  // the arrays' format from here on
   if (to_df) launch_row_sums(dev_mesh(c), c->d_fcsum, c->stream);
   HOFV_CUDA(c, cudaGetLastError());
@@ -865,15 +864,15 @@ int hofv_build_stencils(hofv_ctx* c) {
     HOFV_CUDA(c, cudaMemcpy(c->d_fql, ql.data(), sizeof(int32_t) * nfp, cudaMemcpyHostToDevice));
     if (c->Q == 32) {
       // faces of 8 fan slots (Q = 32): consecutive faces of a tile packed into
-      // groups whose rows with area fill the packed kernel's threads
+      // groups whose points with area fill the packed kernel's threads
       std::vector<int32_t> grp;
       for (int64_t t0 = 0; t0 < c->nfid; t0 += kTile) {
         const int64_t t1 = std::min<int64_t>(t0 + kTile, c->nfid);
         int64_t f = t0;
         while (f < t1) {
-          int rows = 0, n = 0;
-          while (f + n < t1 && n < kPackMaxFaces && rows + ql[f + n] * c->dim <= kPackThreads) {
-            rows += ql[f + n] * c->dim;
+          int points = 0, n = 0;
+          while (f + n < t1 && n < kPackMaxFaces && points + ql[f + n] <= kPackPoints) {
+            points += ql[f + n];
             ++n;
           }
           if (n == 0) return fail(c, HOFV_EINVAL, "a polyhedral face has more points than a packed group");
@@ -1625,13 +1624,20 @@ extern "C" int hofv_newton_solve(hofv_ctx* c, double* u, const hofv_solve_opts* 
   return status;
 }
 
-// host copy of a coefficient array held as double-float pairs -> doubles
-static void df_to_double(std::vector<double>& a) {
-  for (double& x : a) {
-    float hl[2];
-    memcpy(hl, &x, sizeof(hl));
-    x = (double)hl[0] + (double)hl[1];
-  }
+// host copy of a coefficient array held as double-float pairs (two rows a
+// pair of planes) -> doubles [chunk][np][rows]
+static void df_to_double(std::vector<double>& a, int np, int rows) {
+  const std::vector<double> in = a;
+  const float* f = reinterpret_cast<const float*>(in.data());
+  const size_t n = (size_t)np * rows;
+  for (size_t o = 0; o < a.size(); o += n)
+    for (int p = 0; p < np; ++p)
+      for (int i = 0; i < rows; ++i) {
+        const bool odd = (rows & 1) && i == rows - 1;
+        const size_t h = odd ? 2 * (o + (size_t)i * np + p) : 2 * (o + (size_t)(i & ~1) * np + p) + (i & 1);
+        const size_t l = odd ? h + 1 : 2 * (o + (size_t)(i | 1) * np + p) + (i & 1);
+        a[o + (size_t)p * rows + i] = (double)f[h] + (double)f[l];
+      }
 }
 
 extern "C" {
@@ -1653,7 +1659,7 @@ int hofv_get_face_data(hofv_ctx* c, int64_t first, int64_t count, int32_t* stenc
     co.resize((size_t)(t1 - t0) * S * kTile * R);
     HOFV_CUDA(c, cudaMemcpy(co.data(), c->d_fco + t0 * S * kTile * R, sizeof(double) * co.size(),
                             cudaMemcpyDeviceToHost));
-    if (c->prec == HOFV_PREC_DF64) df_to_double(co);
+    if (c->prec == HOFV_PREC_DF64) df_to_double(co, kTile * Q, d);
     if (c->nfd + c->nfy > 0) {
       gc.resize((size_t)(c->nfd + c->nfy) * R);
       HOFV_CUDA(c, cudaMemcpy(gc.data(), c->d_gco, sizeof(double) * gc.size(), cudaMemcpyDeviceToHost));
@@ -1694,7 +1700,7 @@ int hofv_get_cell_data(hofv_ctx* c, int64_t first, int64_t count, int32_t* stenc
     ex.resize((size_t)(t1 - t0) * S * kTile * nlf);
     HOFV_CUDA(c, cudaMemcpy(ex.data(), c->d_cex + t0 * S * kTile * nlf, sizeof(double) * ex.size(),
                             cudaMemcpyDeviceToHost));
-    if (c->prec == HOFV_PREC_DF64) df_to_double(ex);
+    if (c->prec == HOFV_PREC_DF64) df_to_double(ex, kTile, nlf);
   }
   for (int64_t cell = first; cell < hi; ++cell) {
     const int64_t t = cell / kTile - t0, ci = cell % kTile, o = cell - first;
@@ -1964,6 +1970,14 @@ static void tile_rows(const int32_t* rows, int64_t count, int S, std::vector<int
 static int rebuild_from_stencils(hofv_ctx* c) {
   invalidate_graphs(c);
   jv_invalidate(c);
+  if (c->prec == HOFV_PREC_DF64) {
+    // the fits write the coefficients as doubles in their own order: clear
+    // the last tiles, whose slots past the last face or cell they leave alone
+    const size_t ft = (size_t)c->S * kTile * c->Q * c->dim, ct = (size_t)c->S * kTile * c->nlf;
+    if (c->nftile > 0)
+      HOFV_CUDA(c, cudaMemsetAsync(c->d_fco + (c->nftile - 1) * ft, 0, sizeof(double) * ft, c->stream));
+    HOFV_CUDA(c, cudaMemsetAsync(c->d_cex + (c->nctile - 1) * ct, 0, sizeof(double) * ct, c->stream));
+  }
   TRY(run_lsq(c));
   if (c->prec == HOFV_PREC_DF64) TRY(coef_format(c, 1));
   if (c->d_cmass) TRY(run_cell_mass(c));

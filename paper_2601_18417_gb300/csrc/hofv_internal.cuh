@@ -20,7 +20,7 @@ constexpr int kMaxQC = 64;       // Gauss points per cell (4^3)
 constexpr int kPolyMaxSides = 8; // face slots of a polygon cell
 constexpr int kPolyhedronMaxFaces = 16;  // face slots of a polyhedral cell
 constexpr int kPolyFaceMaxCorners = 8;   // corners of a polyhedral face
-constexpr int kPackThreads = 384;        // threads (rows with area) of a packed face group
+constexpr int kPackPoints = 128;         // threads (points with area) of a packed face group
 constexpr int kPackMaxFaces = 8;         // faces of a packed face group
 
 // J^{-1/3} for the neo-Hookean law, with one FP64 correction of a
@@ -80,9 +80,10 @@ struct DevMesh {
   const double* mscale;   // [nc] -rho Omega_P c2, or nullptr (no inertia term)
   const double* cmass;    // [nctile][S][kTile] cell-average weights, or nullptr (ubar = u_P)
   double* inert;          // [dim][nc] scratch: the inertia term of the current call
-  // gradient contraction precision (HOFV_PREC_*).  With HOFV_PREC_DF64 every
-  // 8-byte slot of fco and cex holds a double-float pair (float hi, float lo),
-  // and the state is split into such pairs before the contraction
+  // gradient contraction precision (HOFV_PREC_*).  With HOFV_PREC_DF64 fco and
+  // cex hold double-float pairs (float hi, float lo) by row plane,
+  // [nftile][S][dim][kTile * Q] and [nctile][S][nlf][kTile], and the state is
+  // split into such pairs before the contraction
   int prec;
   float4* su;             // [wst][dim] split state (scratch): (hi, mid, lo, 0) per component
   float4* sv;             // [wst][dim] split Jv direction (scratch)
@@ -90,10 +91,11 @@ struct DevMesh {
   double* vext;           // [dim][wst] extended Jv direction (symmetry faces; scratch)
   // linearisation of the neo-Hookean law at u for the double-float Jv:
   // gradient rows and Gauss-point tractions of every face at u
-  double* gcache;         // [nftile * kTile][R][dim]
-  double* tcache;         // [nftile * kTile][Q][dim]
+  // (by plane, as the pairs)
+  double* gcache;         // [nftile][dim][dim][kTile * Q]
+  double* tcache;         // [nftile][dim][kTile * Q]
   unsigned int* kerr;     // set to 1 by a face kernel whose bounded wait ran out
-  const double* fcsum;    // [nftile * kTile][R] sums over the stencil of the stored
+  const double* fcsum;    // [nftile][dim][kTile * Q] sums over the stencil of the stored
                           // (double-float) gradient coefficients of each row
 };
 
@@ -182,7 +184,7 @@ struct hofv_ctx {
   float4* d_su = nullptr;           // [nc + ng][split4] split state
   float4* d_sv = nullptr;           // [nc + ng][split4] split Jv direction
   double* d_ustar_v = nullptr;      // [nc][nlf][dim]
-  double* d_fcsum = nullptr;        // [nftile * kTile][R] row sums of the stored coefficients
+  double* d_fcsum = nullptr;        // [nftile][dim][kTile * Q] row sums of the stored coefficients
   double* d_vext = nullptr;         // [dim][nc + ng]
   // neo-Hookean double-float Jv: face gradients and tractions at u, valid
   // for the state / residual pair (jv_u, jv_R) while jv_gen == jv_cur
@@ -313,13 +315,14 @@ void launch_jv_df(const DevMesh& m, const Material& mat, const double* v, const 
 // m.tcache
 void launch_jv_cache_fill(const DevMesh& m, const Material& mat, const double* u,
                           const double* ubq, cudaStream_t st);
-// rewrites the n 8-byte slots of a coefficient array in place: to_df != 0
-// turns each double into the double-float pair (float hi, float lo) with
-// hi + lo its value rounded to 48 significant bits; to_df == 0 turns the pairs
-// back into doubles (exactly)
-void launch_coef_format(double* a, int64_t n, int to_df, cudaStream_t st);
-// fcsum[f][r] = sum over the stencil slots of the stored coefficient of face
-// f, row r (double-float pairs summed in FP64, in slot order)
+// rewrites the chunks of a coefficient array in place, each np points of
+// `rows` coefficients: to_df != 0 turns the doubles [np][rows] into the
+// double-float pairs (float hi, float lo) [rows][np] with hi + lo the value
+// rounded to 48 significant bits; to_df == 0 turns the pairs back into
+// doubles (exactly)
+void launch_coef_format(double* a, int64_t chunks, int np, int rows, int to_df, cudaStream_t st);
+// fcsum = sum over the stencil slots of the stored coefficients
+// (double-float pairs summed in FP64, in slot order)
 void launch_row_sums(const DevMesh& m, double* fcsum, cudaStream_t st);
 // raises the dynamic shared-memory limit of the double-float face kernels
 // (once per process, at set-up); 0 or a cudaError_t

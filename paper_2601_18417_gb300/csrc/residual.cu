@@ -639,6 +639,8 @@ void launch_flux_scale(const DevMesh& m, const double* flux, double* out, cudaSt
 // ---------------------------------------------------------------------
 namespace hofv {
 
+__device__ __forceinline__ float2 ld_pair(const float2* __restrict__ pl, int i, int rows, int np);
+
 // tco[tile][N][fi][i][k] from fco[tile][N][fi][q*d + i] and aq
 template <int DIM>
 __global__ void k_build_tco(DevMesh m, double mu, double lam, double* __restrict__ tco) {
@@ -655,12 +657,14 @@ __global__ void k_build_tco(DevMesh m, double mu, double lam, double* __restrict
     for (int k = 0; k < DIM; ++k) T[i][k] = 0.0;
   if (f < m.nfid) {
     const double* co = m.fco + e * m.R;
+    const int np = kTile * m.Q;  // points of the tile: planes of the pairs' layout
+    const float2* pairs = reinterpret_cast<const float2*>(m.fco) + (e - fi) * m.R + fi * m.Q;  // tile, slot
     for (int q = 0; q < m.Q; ++q) {
       double c[DIM], a[DIM], ca = 0.0;
 #pragma unroll
       for (int i = 0; i < DIM; ++i) {
         if (m.prec == HOFV_PREC_DF64) {  // stored as a double-float pair
-          const float2 p = reinterpret_cast<const float2*>(co)[q * DIM + i];
+          const float2 p = ld_pair(pairs + q, i, DIM, np);
           c[i] = (double)p.x + (double)p.y;
         } else {
           c[i] = co[q * DIM + i];
@@ -779,8 +783,9 @@ void launch_tflux(const DevMesh& m, const double* tco, double alpha_kbar, const 
 // same way once per call; each product c u is formed as hi*hi exactly
 // (TwoProduct by FMA, Dekker 1971) plus the cross terms, and accumulated by
 // TwoSum with a compensation float (Dot2, Ogita, Rump & Oishi 2005): twelve
-// FP32 instructions per product.  The sum is converted to FP64 for the law,
-// the quadrature, the stabilisation jump and the assembly, which stay FP64.
+// FP32 operations per product, two products an instruction where they pair.
+// The sum is converted to FP64 for the law, the quadrature, the stabilisation
+// jump and the assembly, which stay FP64.
 //
 // Jv must not difference two residuals contracted separately: each carries
 // an independent rounding of 2^-48 relative, which the division by eps
@@ -790,11 +795,6 @@ void launch_tflux(const DevMesh& m, const double* tco, double alpha_kbar, const 
 // contract v alone and difference the tractions of grad u + eps grad v and
 // grad u in FP64, with grad u and its tractions taken from a cache filled
 // once per linearisation point, so the rounding of grad u cancels exactly.
-//
-// The face kernel keeps several coefficient loads in flight per thread (a
-// register ring) and, in 3-D, runs half a tile per block so that two blocks
-// share an SM and the FP32 contraction of one overlaps the FP64 law of the
-// other.
 // =====================================================================
 namespace hofv {
 
@@ -817,6 +817,67 @@ __device__ __forceinline__ void ff_mac(float ch, float cl, float uh, float ul, f
 }
 
 __device__ __forceinline__ double ff_value(float s, float e) { return (double)s + (double)e; }
+
+// two floats in a 64-bit register: Blackwell's packed FP32 instructions do
+// both halves in one issue slot (the contractions are short of issue slots,
+// not of FP32 lanes)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// ff_mac on both halves, bit for bit (the product is formed negated, which
+// changes no rounding); nch = -ch
+__device__ __forceinline__ void ff_mac2(f32x2 ch, f32x2 nch, f32x2 cl, f32x2 uh, f32x2 ul, f32x2& s,
+                                        f32x2& e) {
+  const f32x2 np = mul2(nch, uh);
+  f32x2 r = fma2(ch, uh, np);
+  r = fma2(ch, ul, r);
+  r = fma2(cl, uh, r);
+  const f32x2 t = sub2(s, np);
+  const f32x2 z = sub2(t, s);
+  const f32x2 q = sub2(sub2(s, sub2(t, z)), add2(np, z));
+  s = t;
+  e = add2(e, add2(q, r));
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+
+// Coefficient pairs of a point's rows are stored two rows together, ready
+// for ff_mac2: plane 2k holds (hi, hi) and plane 2k + 1 (lo, lo) of rows 2k
+// and 2k + 1; an odd last row keeps its plane (hi, lo).  This reads row i of
+// a point whose planes lie np apart.
+__device__ __forceinline__ float2 ld_pair(const float2* __restrict__ pl, int i, int rows, int np) {
+  if ((rows & 1) && i == rows - 1) return pl[(int64_t)i * np];
+  const float2 h = pl[(int64_t)(i & ~1) * np], l = pl[(int64_t)(i | 1) * np];
+  return (i & 1) ? make_float2(h.y, l.y) : make_float2(h.x, l.x);
+}
 
 // split state of cell `id` as double-float pairs (hi, mid): 48 bits
 template <int DIM>
@@ -872,34 +933,52 @@ __device__ __forceinline__ float2 diff3(const float4 x, const float4 r) {
   return make_float2(dh, __fsub_rn(l, __fsub_rn(dh, h)));
 }
 
-__global__ void k_coef_format(double* __restrict__ a, int64_t n, int to_df) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (to_df) {
-      float h, l;
-      split_value(a[i], h, l);
-      const unsigned long long bits =
-          ((unsigned long long)__float_as_uint(l) << 32) | (unsigned long long)__float_as_uint(h);
-      a[i] = __longlong_as_double((long long)bits);
-    } else {
-      const float2 p = reinterpret_cast<const float2*>(a)[i];
-      a[i] = ff_value(p.x, p.y);
+// Coefficient arrays in place between doubles and double-float pairs.  An
+// array is a list of chunks (one tile and stencil slot each) of np points
+// (face Gauss points, or cells) with `rows` coefficients a point: doubles as
+// [np][rows], pairs as planes [rows][np] (ld_pair), so that a thread that
+// takes a point reads its rows coalesced with its neighbours'.  One block a
+// chunk.
+__global__ void __launch_bounds__(256) k_coef_format(double* __restrict__ a, int np, int rows, int to_df) {
+  extern __shared__ double2 chunk_raw[];
+  double* chunk = reinterpret_cast<double*>(chunk_raw);
+  const int n = np * rows;
+  double* g = a + (int64_t)blockIdx.x * n;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) chunk[k] = g[k];
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    if (to_df) {  // k = plane * np + point
+      const int pl = k / np;
+      const double* c = chunk + (k % np) * rows;
+      float2 v;
+      if ((rows & 1) && pl == rows - 1) {
+        split_value(c[pl], v.x, v.y);
+      } else {
+        float h0, l0, h1, l1;
+        split_value(c[pl & ~1], h0, l0);
+        split_value(c[pl | 1], h1, l1);
+        v = (pl & 1) ? make_float2(l0, l1) : make_float2(h0, h1);
+      }
+      reinterpret_cast<float2*>(g)[k] = v;
+    } else {  // k = point * rows + i
+      const float2 p = ld_pair(reinterpret_cast<const float2*>(chunk) + k / rows, k % rows, rows, np);
+      g[k] = ff_value(p.x, p.y);
     }
   }
 }
 
-// fcsum[f][r] = sum_n of the stored pair of face f, row r, slot n
+// fcsum[tile][i][point] = sum_n of the stored pairs of row i of the point
 __global__ void k_row_sums(DevMesh m, double* __restrict__ fcsum) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (face, row)
-  const int R = m.R;
-  if (e >= m.nftile * kTile * R) return;
-  const int64_t tile = e / (kTile * R);
-  const int k = (int)(e % (kTile * R));  // fi * R + r within the tile
-  const float2* co = reinterpret_cast<const float2*>(m.fco) + tile * (int64_t)m.S * kTile * R + k;
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (tile, row, point)
+  const int np = kTile * m.Q, cs = kTile * m.R;
+  if (e >= m.nftile * cs) return;
+  const int64_t tile = e / cs;
+  const int i = (int)(e % cs) / np, p = (int)(e % cs) % np;
+  const float2* co = reinterpret_cast<const float2*>(m.fco) + tile * (int64_t)m.S * cs + p;
   double sum = 0.0;
   for (int n = 0; n < m.S; ++n) {
-    const float2 p = co[(int64_t)n * kTile * R];
-    sum += ff_value(p.x, p.y);
+    const float2 c = ld_pair(co + (int64_t)n * cs, i, m.dim, np);
+    sum += ff_value(c.x, c.y);
   }
   fcsum[e] = sum;
 }
@@ -909,42 +988,126 @@ void launch_row_sums(const DevMesh& m, double* fcsum, cudaStream_t st) {
   if (n > 0) k_row_sums<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m, fcsum);
 }
 
-void launch_coef_format(double* a, int64_t n, int to_df, cudaStream_t st) {
-  if (n <= 0) return;
-  const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, int64_t{1} << 16);  // grid-stride
-  k_coef_format<<<g, 256, 0, st>>>(a, n, to_df);
+void launch_coef_format(double* a, int64_t chunks, int np, int rows, int to_df, cudaStream_t st) {
+  if (chunks <= 0) return;
+  k_coef_format<<<(unsigned)chunks, 256, sizeof(double) * np * rows, st>>>(a, np, rows, to_df);
 }
 
-// stabilisation extrapolation of the state w (split sw), one thread per
-// (cell, local face): out[(cell * NLF + lf) * DIM + j] = w_P + sum_N e_N w_N
+// Stabilisation extrapolation of the state w (split sw):
+//   out[(cell * NLF + lf) * DIM + j] = w_P + sum_N e_N w_N.
+// A block takes a tile of 32 cells, lane = cell.  A warp takes RPG of the
+// cells' rows and every W-th stencil slot: each gathered value serves RPG
+// rows, and the slots of a cell are spread over W warps, so that a mesh of a
+// few tiles still keeps its loads in flight.  The warps' partial sums meet in
+// shared memory as float pairs and are added in a fixed order.  Rows without
+// a flux (polygon and polyhedron slots past a cell's last face, traction
+// faces) are never read back and, where slots may be empty, load nothing.
+// Measured (us, one thread a (cell, face) -> this): 13^3 hexes p = 3 60 -> 25
+// (four warps a tile hide each other's latency), 48^3 hexes p = 3 187 -> 137
+// (0.55 of HBM: the gathers and the packed products), p = 2 148 -> 111, 512^2
+// quads p = 3 76 -> 66, 24-layer prisms 58 -> 48, 6 17^3 tetrahedra 54 -> 31.
+template <int NLF>
+struct UsShape {
+  static constexpr int RPG = NLF >= 8 ? 4 : NLF;   // rows a warp takes
+  static constexpr int NG = NLF / RPG;             // row groups
+  static constexpr bool SPARSE = NLF >= 8;         // cells with empty face slots
+  static constexpr int split(int S) { return NLF == 16 ? 2 : S > 32 ? 4 : 2; }
+  static constexpr int THREADS = NLF >= 8 ? 256 : 128;  // at most
+};
+
 template <int DIM, int NLF>
-__global__ void __launch_bounds__(32 * NLF)
+__global__ void __launch_bounds__(UsShape<NLF>::THREADS, 512 / UsShape<NLF>::THREADS)
     k_ustar_df(DevMesh m, const float4* __restrict__ sw, const double* __restrict__ w,
                double* __restrict__ out) {
+  using SH = UsShape<NLF>;
+  constexpr int RPG = SH::RPG, NP = RPG / 2, NV = NLF * DIM, U = 4;
+  constexpr bool ODD = RPG & 1;
+  extern __shared__ float2 part[];     // [W][NV][33]
+  const int S = m.S;
   const int64_t tile = blockIdx.x;
-  const int it = threadIdx.x;  // ci * NLF + lf
-  const int ci = it / NLF;
-  const int64_t cell = tile * kTile + ci;
-  const int32_t* __restrict__ st = m.cst + tile * m.S * kTile + ci;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int W = (blockDim.x >> 5) / SH::NG, g = wid / W, k = wid % W;
+  const int64_t cell = tile * kTile + lane;
+  const int32_t* __restrict__ st = m.cst + tile * (int64_t)S * kTile + lane;
   const float2* __restrict__ ex =
-      reinterpret_cast<const float2*>(m.cex) + tile * (int64_t)m.S * kTile * NLF + it;
-  float s[DIM], e[DIM];
+      reinterpret_cast<const float2*>(m.cex) + tile * (int64_t)S * kTile * NLF + g * RPG * kTile + lane;
+  unsigned live = ~0u;                 // bit r: rows 2r, 2r + 1 are needed
+  if (SH::SPARSE) {
+    live = 0;
+    if (cell < m.nc)
 #pragma unroll
-  for (int j = 0; j < DIM; ++j) s[j] = e[j] = 0.f;
-#pragma unroll 4
-  for (int n = 0; n < m.S; ++n) {
-    const int32_t id = __ldg(st + n * kTile);
-    const float2 c = __ldg(ex + (int64_t)n * kTile * NLF);
-    float h[DIM], l[DIM];
-    ld_split<DIM>(sw, id, h, l);
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) ff_mac(c.x, c.y, h[j], l[j], s[j], e[j]);
+      for (int r = 0; r < RPG; ++r)
+        if (__ldg(m.cface + cell * NLF + g * RPG + r) != 0) live |= 1u << (r / 2);
   }
-  if (cell < m.nc) {
-    const int64_t ws = m.wst;
-    const int64_t o = (cell * NLF + (it % NLF)) * DIM;
+  f32x2 s[NP][DIM], e[NP][DIM];
+  float so[DIM], eo[DIM];              // an odd last row
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) out[o + j] = w[j * ws + cell] + ff_value(s[j], e[j]);
+  for (int j = 0; j < DIM; ++j) {
+    so[j] = eo[j] = 0.f;
+#pragma unroll
+    for (int r = 0; r < NP; ++r) s[r][j] = e[r][j] = 0;
+  }
+  int32_t id[U];
+#pragma unroll
+  for (int d = 0; d < U; ++d) id[d] = k + d * W < S ? __ldg(st + (k + d * W) * kTile) : 0;
+  for (int n0 = k; n0 < S; n0 += U * W) {
+    float2 c[U][RPG], u[U][DIM];
+#pragma unroll
+    for (int d = 0; d < U; ++d) {
+      const int n = n0 + d * W;
+#pragma unroll
+      for (int r = 0; r < RPG; ++r)
+        c[d][r] = n < S && (live >> (r / 2) & 1) ? __ldg(ex + ((int64_t)n * NLF + r) * kTile)
+                                                 : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < DIM; ++j)
+        u[d][j] = __ldg(reinterpret_cast<const float2*>(sw + (int64_t)id[d] * DIM + j));
+    }
+#pragma unroll
+    for (int d = 0; d < U; ++d) {
+      const int n = n0 + (U + d) * W;
+      id[d] = n < S ? __ldg(st + n * kTile) : 0;
+    }
+#pragma unroll
+    for (int d = 0; d < U; ++d) {
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) {
+        const f32x2 uh = pack2(u[d][j].x, u[d][j].x), ul = pack2(u[d][j].y, u[d][j].y);
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+          const f32x2 ch = pack2(c[d][2 * r].x, c[d][2 * r].y);
+          ff_mac2(ch, neg2(ch), pack2(c[d][2 * r + 1].x, c[d][2 * r + 1].y), uh, ul, s[r][j], e[r][j]);
+        }
+        if (ODD) ff_mac(c[d][RPG - 1].x, c[d][RPG - 1].y, u[d][j].x, u[d][j].y, so[j], eo[j]);
+      }
+    }
+  }
+  {
+    float2* p = part + ((int64_t)k * NV + g * RPG * DIM) * 33 + lane;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+#pragma unroll
+      for (int r = 0; r < NP; ++r) {
+        const float2 a = unpack2(s[r][j]), b = unpack2(e[r][j]);
+        p[(2 * r * DIM + j) * 33] = make_float2(a.x, b.x);
+        p[((2 * r + 1) * DIM + j) * 33] = make_float2(a.y, b.y);
+      }
+      if (ODD) p[((RPG - 1) * DIM + j) * 33] = make_float2(so[j], eo[j]);
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < kTile * NV; t += blockDim.x) {
+    const int ci = t / NV, v = t % NV;
+    const int64_t c = tile * kTile + ci;
+    if (c >= m.nc) break;
+    float2 a = part[v * 33 + ci];
+    for (int q = 1; q < W; ++q) {
+      const float2 b = part[(q * NV + v) * 33 + ci];
+      float h, l;
+      two_sum(a.x, b.x, h, l);
+      a = make_float2(h, __fadd_rn(l, __fadd_rn(a.y, b.y)));
+    }
+    out[c * NV + v] = w[(v % DIM) * m.wst + c] + ff_value(a.x, a.y);
   }
 }
 
@@ -958,36 +1121,12 @@ __device__ __forceinline__ double mirror_i(const double* x, const double* n, int
   return x[i] - 2.0 * un * n[i];
 }
 
-// 16-byte asynchronous copy global -> shared (sm_80 and later), for gathers
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
-}
-// n doubles (n even, both ends 16-byte aligned) global -> shared, by the
-// block's nthreads threads
-__device__ __forceinline__ void stage16(double* dst, const double* src, int n, int it, int nthreads) {
-  for (int c = it; c < n / 2; c += nthreads) cp_async16(dst + 2 * c, src + 2 * c);
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// wait until at most N of this thread's committed groups are pending
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Face fluxes, double-float gradient rows.  QD Gauss points per face
-// (R = QD * DIM rows), FPB faces per block (BPT = 32 / FPB blocks per tile),
-// blockDim = FPB * R; sw is the three-float split of the state contracted
-// (u, or v in the Jv modes), wd the same state in FP64 and ws its
-// extrapolated values.
+// Face fluxes, double-float gradient rows.  One thread takes one Gauss point
+// of one face: its DIM coefficient rows (DIM x DIM products a stencil cell),
+// then the law at that point in registers; the tractions meet in shared
+// memory only for the sum over the face.  QD points a face, FPB consecutive
+// faces a block (a group may span two tiles); sw is the three-float split of the state contracted (u, or v in the Jv modes), wd
+// the same state in FP64 and ws its extrapolated values.
 //
 // Each gradient is contracted against the differences to a reference cell,
 // the face's nearest stencil cell N0:
@@ -998,539 +1137,324 @@ __device__ __forceinline__ void cp_async_wait_group() {
 // magnitude), and the last term is one FP64 product with the FP64 row sum
 // of the stored coefficients.  The stored pairs differ from the FP64
 // coefficients by up to 2^-48 of each; through the row sum that difference
-// still meets w_N0 itself (the sum of the pairs, not of the originals).  The block first gathers its faces' stencil
-// cells' splits into shared memory (16-byte asynchronous copies, [S][FPB]
-// entries) and turns each into the double-float difference to its face's
-// reference (exact differences of the splits); the contraction then reads
-// them from shared memory (the R threads of a face share each entry) and
-// skips the reference itself, whose difference is zero: its coefficient
-// enters only through the row sum and is never read.  Each
-// thread streams its coefficient row through a ring of RING registers: the
-// coefficient of slot n + RING is requested when slot n is consumed, keeping
-// RING coalesced 8-byte loads in flight per thread; with R a compile-time
-// constant every ring offset is an immediate.  Faces come in groups of part
-// of a tile, one thread per (face, row): in 3-D a quarter tile of 216
-// threads for 3 x 3 points, five blocks an SM (measured on the 128^3
-// neo-Hookean block: quarter tiles 7 % faster than half tiles two an SM,
-// 10 % faster than eighth tiles), half tiles otherwise, and for faces with
-// many points (polyhedral fans, R = 48 or 96) quarter or eighth tiles of 384
-// threads.  For 3 x 3 points the operands read after the contraction (row
-// sums, reference values, area vectors, the Jv cache) are copied into shared
-// memory while it runs.
-// A block contracts GPB groups one after the other (the gradients stay in
-// shared memory) and then evaluates the law at all their Gauss points at
-// once: R = Q d rows a face, so d groups have exactly as many points as the
-// block has threads and the FP64 law runs on full warps.
-// Rows of points without area (polyhedral fan slots past a face's last
-// corner) load nothing.
-template <int DIM, int QD>
+// still meets w_N0 itself (the sum of the pairs, not of the originals).
+// The block first forms its faces' differences (exact differences of the
+// splits) in shared memory, slots 1 .. S-1; the reference's own difference
+// is zero and its coefficient enters only through the row sum.  Each thread
+// then streams its DIM rows through a ring of RING slots in registers: the
+// coefficients of slot n + RING are requested when slot n is consumed.  The
+// pairs are stored by plane (k_coef_format), so every request of a warp is
+// 256 contiguous bytes.
+// Points without area (polyhedral fan slots past a face's last corner) load
+// nothing.
+//
+// PACK: polyhedral faces of 8 fan slots (QD = 32).  A group is a run of
+// consecutive faces of one tile whose points with area fill the block's
+// kPackPoints threads (at most kPackMaxFaces faces; the host builds the runs,
+// DevMesh::pgrp); thread it takes the group's it-th point with area.
+// What bounds it and what was measured (GB300, 2070 MHz; us of the kernel in
+// a Jacobian-vector product: one thread a coefficient row before -> this):
+// 48^3 hexes p = 3 neo-Hookean 1554 -> 1132, 48^3 hexes p = 2 807 -> 502,
+// 512^2 quads p = 3 linear 197 -> 129, 24-layer prisms 524 -> 344, 6 17^3
+// tetrahedra 158 -> 104.  The coefficient stream is 85 % of measured HBM at
+// p = 3; the rest is the FP64 law (without it: 1009 of 1266 us at that stage)
+// and, at p = 2, the gather of the differences (442 of 582 us without).
+//  * A thread a point instead of a row: a difference read from shared memory
+//    serves DIM rows, the gradient never leaves registers, and no barrier
+//    stands between contraction and law, so one warp's FP64 law runs beside
+//    other warps' contraction.
+//  * Small groups (14 faces of 9 points fill 126 of 128 threads; 16 faces of
+//    4): the phases of more blocks mix.  32 faces a block, two an SM: 1657 us;
+//    16 faces (144 of 160 threads): 1423; 14: 1383.
+//  * AHEAD: the pairs of slot n + RING + AHEAD are prefetched into L2, so the
+//    ring only has to cover an L2 hit, and five blocks an SM fit in registers:
+//    1383 -> 1270 us (4 to 16 slots ahead alike; 2-D 4, of its 19 slots).
+//  * Packed FP32 instructions (ff_mac2): 1266 -> 1155 us at p = 3, 582 -> 500
+//    at p = 2, 147 -> 129 on the quads.
+//  * A ring of 4 (3 in 2-D, whose twelve blocks an SM need 56 registers);
+//    ten stencil cells' ids of a thread loaded before their values: 3 %.
+// Not kept: the pair widened to double by integer operations (1 % slower),
+// the operands of the law prefetched at the start (no gain).
+template <int DIM, int QD, bool PACK>
 struct DfShape {
-  static constexpr int FPB = DIM == 2  ? 32
-                             : QD == 9  ? 8
+  static constexpr int FPB = PACK       ? kPackMaxFaces
+                             : DIM == 2 ? 32
+                             : QD == 1  ? 32
+                             : QD == 9  ? 14
                              : QD == 16 ? 8
-                             : QD == 32 ? 4
                                         : 16;  // faces per group
-  // coefficient loads in flight per thread (4 in 2-D: 6 % slower; 3 x 3
-  // points: 6, with five blocks an SM, 5 % faster than 8 with four)
-  static constexpr int RING = (DIM == 3 && QD == 9) ? 6 : 8;
-  static constexpr int THREADS = FPB * QD * DIM;
-  // face groups per block: with GPB = d, GPB FPB Q = THREADS and each thread
-  // evaluates one law (a face's Gauss point) after the block's contractions
-  // (measured: 9 % faster on the 48-layer prisms, 5 % on 512^2 quads); 3 x 3
-  // points keep one group a block (5 % slower with three on the 128^3 block)
-  static constexpr int GPB = (DIM == 3 && QD == 9) ? 1 : DIM;
-  static constexpr int MIN_BLOCKS = DIM == 2 ? 6 : (THREADS <= 256 ? 5 : 2);  // per SM
-  // 3 x 3 points: the epilogue's and the law's operands (row sums, reference
-  // values, area vectors and, in Jv mode, the cached gradients and
-  // tractions) are copied into shared memory while the contraction runs (a
-  // second group of asynchronous copies, waited for after it), instead of
-  // being loaded after it with their latency exposed (measured: 5 % faster
-  // on the 128^3 block; 27 % slower with 2 x 2 points, three groups a block)
-  static constexpr bool STAGE = DIM == 3 && QD == 9;
+  static constexpr int THREADS = PACK ? kPackPoints : (FPB * QD + 31) / 32 * 32;
+  static constexpr int RING = DIM == 2 ? 3 : 4;    // slots requested ahead in registers
+  static constexpr int AHEAD = DIM == 2 ? 4 : 8;   // ... and beyond them into L2
+  static constexpr int IDS = DIM == 2 ? 7 : 10;    // stencil ids of a thread loaded together
+  static constexpr int BLOCKS = (DIM == 2 ? 1152 : PACK || QD == 9 ? 640 : 512) / THREADS;
+  static constexpr int MIN_BLOCKS = BLOCKS < 32 ? BLOCKS : 32;  // an SM holds 32 at most
 };
 
-// dynamic shared memory: the gathered cell values and the faces' references
-// (one group at a time), then the gradients and tractions of all groups
-template <int DIM, int QD>
+// dynamic shared memory: the differences (DIM pairs a slot and face), the
+// tractions of the block's points
+template <int DIM, int QD, bool PACK>
 static size_t df_smem_bytes(int S) {
-  using SH = DfShape<DIM, QD>;
-  constexpr int R = QD * DIM;
-  const size_t gath = (size_t)S * SH::FPB * DIM * 16;
-  const size_t law = (size_t)SH::GPB * SH::FPB * (R * DIM + QD * DIM) * sizeof(double);
-  const size_t staged = SH::STAGE ? (size_t)SH::GPB * SH::FPB * (QD * 3 + R + DIM) * sizeof(double) : 0;
-  return gath + law + staged;
+  using SH = DfShape<DIM, QD, PACK>;
+  return (size_t)(S - 1) * SH::FPB * DIM * 8 + sizeof(double) * SH::THREADS * DIM;
 }
 
-template <int DIM, int LAW, int MODE, int QD>
-__global__ void __launch_bounds__(DfShape<DIM, QD>::THREADS, DfShape<DIM, QD>::MIN_BLOCKS)
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+template <int DIM, int LAW, int MODE, int QD, bool PACK>
+__global__ void __launch_bounds__(DfShape<DIM, QD, PACK>::THREADS, DfShape<DIM, QD, PACK>::MIN_BLOCKS)
     k_flux_df(DevMesh m, Material mt, const float4* __restrict__ sw, const double* __restrict__ wd,
               const double* __restrict__ ws, const double* __restrict__ ubq,
               const double* __restrict__ ubf, const double* __restrict__ d_eps,
               double* __restrict__ flux) {
-  using SH = DfShape<DIM, QD>;
-  constexpr int FPB = SH::FPB, BPT = kTile / FPB, GPB = SH::GPB, Q = QD, R = QD * DIM;
-  constexpr int kRing = SH::RING;
-  constexpr int CS = kTile * R;  // coefficient stride between stencil slots
+  using SH = DfShape<DIM, QD, PACK>;
+  constexpr int FPB = SH::FPB, T = SH::THREADS, Q = QD, K = SH::RING;
+  constexpr int NP = kTile * Q;        // points of a tile: plane stride of the coefficients
+  constexpr int CS = NP * DIM;         // coefficient stride between stencil slots
   extern __shared__ __align__(16) double sm[];
   const int S = m.S;
-  // [S][FPB][DIM] gathered values of one group; slots 1.. then hold the
-  // differences to slot 0, the faces' reference cells (zero difference)
-  float4* us = reinterpret_cast<float4*>(sm);
-  double* Gs = reinterpret_cast<double*>(us + (size_t)S * FPB * DIM);  // [GPB][FPB][R][DIM]
-  double* Ts = Gs + GPB * FPB * R * DIM;                               // [GPB][FPB][Q][DIM]
-  constexpr bool STG = SH::STAGE;
-  double* As = Ts + GPB * FPB * Q * DIM;  // [GPB][FPB][Q][3] staged area vectors
-  double* Cs = As + GPB * FPB * Q * 3;    // [GPB][FPB][R] staged row sums
-  double* Ws = Cs + GPB * FPB * R;        // [GPB][FPB][DIM] staged reference values
-  const int64_t ldw = m.wst;
-  const int64_t ngroups = m.nftile * BPT;
-  const int64_t g0 = (int64_t)blockIdx.x * GPB;
-  const int ng = (int)(ngroups - g0 < GPB ? ngroups - g0 : GPB);  // the same for every thread
+  float4* ua = reinterpret_cast<float4*>(sm);                            // [S-1][FPB] components 0, 1
+  float2* ub = reinterpret_cast<float2*>(ua + (size_t)(S - 1) * FPB);    // [S-1][FPB] component 2
+  double* Ts = reinterpret_cast<double*>(ub + (DIM == 3 ? (size_t)(S - 1) * FPB : 0));  // [T][DIM]
+  __shared__ int rowp[PACK ? FPB + 1 : 1];  // points with area before each face of the group
   const int it = threadIdx.x;
-  const double eps = MODE == kDfJv ? __ldg(d_eps) : 0.0;
-  const int fi = it / R, r = it % R;
-  float2 cq[kRing];
-  for (int gi = 0; gi < ng; ++gi) {
-    const int64_t grp = g0 + gi;
-    const int64_t tile = grp / BPT;
-    const int fb = (int)(grp % BPT) * FPB;  // first face of the group within its tile
-    const int64_t f0 = tile * kTile + fb;
-    const int64_t f = f0 + fi;
-    const int32_t* __restrict__ st = m.fst + tile * (int64_t)S * kTile + fb;
-    const float2* __restrict__ co =
-        reinterpret_cast<const float2*>(m.fco) + tile * (int64_t)S * CS + fb * R + it;
-    // rows of points without area (polyhedral fan slots past a face's last
-    // corner) read no coefficient and keep a zero gradient
-    const bool live = m.fql == nullptr || r < __ldg(m.fql + f) * DIM;
-    // stencil slots this thread contracts: 1 .. S-1 (slot 0, the reference,
-    // enters only through the row sums)
-    const int SL = live ? S - 1 : 0;
-    co += CS;  // coefficients of slot 1
-    // the first coefficients of the ring, then the gather of the cell values
-#pragma unroll
-    for (int d = 0; d < kRing; ++d) cq[d] = d < SL ? __ldg(co + d * CS) : make_float2(0.f, 0.f);
-    for (int t = it; t < S * FPB; t += SH::THREADS) {
-      const int n = t / FPB, fj = t % FPB;
-      const int32_t id = __ldg(st + n * kTile + fj);
-#pragma unroll
-      for (int h = 0; h < DIM; ++h) cp_async16(us + t * DIM + h, sw + (int64_t)id * DIM + h);
-      if (STG && n == 0) {  // the reference cell's FP64 value
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) cp_async8(Ws + (gi * FPB + fj) * DIM + j, wd + j * ldw + id);
-      }
-    }
-    cp_async_commit();
-    if (STG) {
-      // second group, waited for only after the contraction: each thread's
-      // own row sum and (Jv) cached gradient row, and the group's area
-      // vectors and (Jv) cached tractions for the law
-      cp_async8(Cs + gi * FPB * R + it, m.fcsum + f * R + r);
-      if (MODE == kDfJv) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j)
-          cp_async8(Gs + (gi * FPB * R + it) * DIM + j, m.gcache + (f * R + r) * DIM + j);
-        stage16(Ts + gi * FPB * Q * DIM, m.tcache + f0 * Q * DIM, FPB * Q * DIM, it, SH::THREADS);
-      }
-      // area vectors: faces up to the last one stored
-      const int na = (int)(m.nf - f0 < FPB ? (m.nf - f0 > 0 ? m.nf - f0 : 0) : FPB) * Q * 3;
-      for (int c = it; c < na; c += SH::THREADS) cp_async8(As + gi * FPB * Q * 3 + c, m.aq + f0 * Q * 3 + c);
-      cp_async_commit();
-      cp_async_wait_group<1>();  // the gather
-    } else {
-      cp_async_wait_group<0>();
+  int64_t f0;
+  int nf;                              // faces of the group
+  int fi = it / Q, q = it % Q;         // this thread's face in the group and its point
+  bool live;
+  if (PACK) {
+    f0 = m.pgrp[2 * (int64_t)blockIdx.x];
+    nf = m.pgrp[2 * (int64_t)blockIdx.x + 1];
+    if (it == 0) {
+      int acc = 0;
+      rowp[0] = 0;
+      for (int k = 0; k < FPB; ++k) rowp[k + 1] = acc += k < nf ? m.fql[f0 + k] : 0;
     }
     __syncthreads();
-    for (int t = FPB * DIM + it; t < S * FPB * DIM; t += SH::THREADS) {
-      const float2 dv = diff3(us[t], us[t % (FPB * DIM)]);
-      us[t] = make_float4(dv.x, dv.y, 0.f, 0.f);
-    }
-    __syncthreads();
-    // (1) gradient rows: thread (fi, r) accumulates sum_N c_{r,N} (w_N - w_N0)
-    float s[DIM], e[DIM];
+    fi = 0;
+    while (fi + 1 < nf && rowp[fi + 1] <= it) ++fi;
+    live = it < rowp[nf];
+    q = live ? it - rowp[fi] : 0;
+  } else {
+    f0 = (int64_t)blockIdx.x * FPB;
+    nf = (int)(m.nfid - f0 < FPB ? m.nfid - f0 : FPB);
+    live = fi < nf && (m.fql == nullptr || q < __ldg(m.fql + f0 + fi));
+    if (fi >= nf) fi = 0;
+  }
+  const int64_t f = f0 + fi;
+  const int64_t tile = f / kTile;
+  const int pt = (int)(f % kTile) * Q + q;  // point within the tile
+  const float2* __restrict__ co =
+      reinterpret_cast<const float2*>(m.fco) + tile * (int64_t)S * CS + CS + pt;  // slot 1
+  const int SL = live ? S - 1 : 0;     // stencil slots this thread contracts: 1 .. S-1
+  float2 cq[K][DIM];
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) s[j] = e[j] = 0.f;
-    const float4* __restrict__ uf = us + FPB * DIM + fi * DIM;  // slot 1 of the thread's face
-    auto mac_slot = [&](int n, float2 c) {
+  for (int d = 0; d < K; ++d)
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+      cq[d][i] = d < SL ? __ldg(co + d * CS + i * NP) : make_float2(0.f, 0.f);
+  constexpr int PD = SH::AHEAD;
+#pragma unroll
+  for (int d = K; d < K + PD; ++d)
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+      if (d < SL) prefetch_l2(co + d * CS + i * NP);
+  // the group's differences; a thread keeps one face, STEP slots at a time
+  {
+    constexpr int STEP = T / FPB, IDB = SH::IDS;
+    const int fj = it % FPB;
+    if (fj < nf && it < STEP * FPB) {
+      const int64_t fg = f0 + fj;
+      const int32_t* __restrict__ st = m.fst + fg / kTile * (int64_t)S * kTile + fg % kTile;
+      float4 r[DIM];
+      const int32_t id0 = __ldg(st);
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) r[j] = __ldg(sw + (int64_t)id0 * DIM + j);
+      for (int n0 = 1 + it / FPB; n0 < S; n0 += IDB * STEP) {
+        int32_t id[IDB];  // the cells first: one wait for their list, one for their values
+#pragma unroll
+        for (int k = 0; k < IDB; ++k) id[k] = n0 + k * STEP < S ? __ldg(st + (n0 + k * STEP) * kTile) : 0;
+#pragma unroll
+        for (int k = 0; k < IDB; ++k) {
+          const int n = n0 + k * STEP;
+          if (n >= S) break;
+          float4 x[DIM];
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) x[j] = __ldg(sw + (int64_t)id[k] * DIM + j);
+          const float2 a = diff3(x[0], r[0]), b = diff3(x[1], r[1]);
+          ua[(n - 1) * FPB + fj] = make_float4(a.x, b.x, a.y, b.y);
+          if constexpr (DIM == 3) ub[(n - 1) * FPB + fj] = diff3(x[2], r[2]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // gradient rows: sum_N c_{i,N} (w_N - w_N0), rows 0 and 1 together for each
+  // component; in 3-D row 2 takes components 0 and 1 together, then 2 alone
+  f32x2 s01[DIM], e01[DIM], s2 = 0, e2 = 0;
+  float s22 = 0.f, e22 = 0.f;
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) s01[j] = e01[j] = 0;
+  auto mac_slot = [&](int n, const float2 (&c)[DIM]) {
+    const float4 a = ua[n * FPB + fi];  // (hi, hi, lo, lo) of components 0, 1
+    const f32x2 ch = pack2(c[0].x, c[0].y), cl = pack2(c[1].x, c[1].y), nch = neg2(ch);
+    ff_mac2(ch, nch, cl, pack2(a.x, a.x), pack2(a.z, a.z), s01[0], e01[0]);
+    ff_mac2(ch, nch, cl, pack2(a.y, a.y), pack2(a.w, a.w), s01[1], e01[1]);
+    if constexpr (DIM == 3) {
+      const float2 b = ub[n * FPB + fi];
+      ff_mac2(ch, nch, cl, pack2(b.x, b.x), pack2(b.y, b.y), s01[2], e01[2]);
+      const f32x2 c2 = pack2(c[2].x, c[2].x);
+      ff_mac2(c2, neg2(c2), pack2(c[2].y, c[2].y), pack2(a.x, a.y), pack2(a.z, a.w), s2, e2);
+      ff_mac(c[2].x, c[2].y, b.x, b.y, s22, e22);
+    }
+  };
+  int n0 = 0;
+  // steady part: every request in range
+  for (; n0 + 2 * K <= SL; n0 += K) {
+    const float2* cn = co + (int64_t)(n0 + K) * CS;
+#pragma unroll
+    for (int d = 0; d < K; ++d) {
+      float2 c[DIM];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        c[i] = cq[d][i];
+        cq[d][i] = __ldg(cn + d * CS + i * NP);
+      }
+      const float2* pf = co + (int64_t)min(n0 + d + K + PD, SL - 1) * CS;
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) prefetch_l2(pf + i * NP);
+      mac_slot(n0 + d, c);
+    }
+  }
+  // the operands of what follows are requested while the last slots run
+  const int64_t tp = tile * NP;        // first point of the tile in the per-point arrays
+  double cs[DIM], w0[DIM], a[3];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) cs[i] = w0[i] = a[i] = 0.0;
+  if (live) {
+    const int32_t id0 = __ldg(m.fst + tile * (int64_t)S * kTile + f % kTile);
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      cs[i] = __ldg(m.fcsum + tp * DIM + i * NP + pt);
+      a[i] = __ldg(m.aq + (f * Q + q) * 3 + i);
+      w0[i] = __ldg(wd + i * m.wst + id0);
+    }
+  }
+  // the last K .. 2 K - 1 slots (fewer if S <= K)
+#pragma unroll
+  for (int d = 0; d < K; ++d) {
+    const int n = n0 + d;
+    if (n < SL) {
+      float2 c[DIM];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i) {
+        c[i] = cq[d][i];
+        if (n + K < SL) cq[d][i] = __ldg(co + (int64_t)(n + K) * CS + i * NP);
+      }
+      mac_slot(n, c);
+    }
+  }
+  double gu[DIM][DIM], tu[DIM];        // the linearisation (Jv)
+  if (MODE == kDfJv && live) {
+#pragma unroll
+    for (int i = 0; i < DIM; ++i) {
+      tu[i] = m.tcache[tp * DIM + i * NP + pt];
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) gu[i][j] = m.gcache[(tp * DIM + i * NP) * DIM + j * NP + pt];
+    }
+  }
+#pragma unroll
+  for (int d = 0; d < K; ++d)
+    if (n0 + K + d < SL) mac_slot(n0 + K + d, cq[d]);
+  float s[DIM][DIM], e[DIM][DIM];
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) {
+    const float2 a = unpack2(s01[j]), b = unpack2(e01[j]);
+    s[0][j] = a.x, s[1][j] = a.y, e[0][j] = b.x, e[1][j] = b.y;
+  }
+  if constexpr (DIM == 3) {
+    const float2 a = unpack2(s2), b = unpack2(e2);
+    s[2][0] = a.x, s[2][1] = a.y, s[2][2] = s22;
+    e[2][0] = b.x, e[2][1] = b.y, e[2][2] = e22;
+  }
+  double t[DIM];
+#pragma unroll
+  for (int i = 0; i < DIM; ++i) t[i] = 0.0;
+  if (live) {
+    const double eps = MODE == kDfJv ? __ldg(d_eps) : 0.0;
+    double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)  // + w_N0 sum_N c_N, in FP64
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) G[i][j] = fma(cs[i], w0[j], ff_value(s[i][j], e[i][j]));
+    if (MODE == kDfResidual || MODE == kDfFill) {
+      if (f >= m.nfi && f < m.nfi + m.nfd) {  // ghost node of a displacement face (prescribed data)
+        const int64_t fd = f - m.nfi;
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) {
+          const double cg = m.gco[(fd * Q + q) * DIM + i];
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) G[i][j] = fma(cg, ubq[(fd * Q + q) * DIM + j], G[i][j]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        const float4 a = uf[n * FPB * DIM + j];
-        ff_mac(c.x, c.y, a.x, a.y, s[j], e[j]);
+        if (MODE == kDfFill) m.gcache[(tp * DIM + i * NP) * DIM + j * NP + pt] = G[i][j];
+        if (MODE == kDfJv) G[i][j] = fma(eps, G[i][j], gu[i][j]);  // grad (u + eps v)
       }
-    };
-    int n0 = 0;
-    // steady part: every request in range
-    for (; n0 + 2 * kRing <= SL; n0 += kRing) {
-      const float2* cn = co + (n0 + kRing) * CS;
+    traction<DIM, LAW>(G, a, mt, t);
 #pragma unroll
-      for (int d = 0; d < kRing; ++d) {
-        const float2 c = cq[d];
-        cq[d] = __ldg(cn + d * CS);
-        mac_slot(n0 + d, c);
-      }
-    }
-    // the last kRing .. 2 kRing - 1 slots (fewer if S < kRing)
-#pragma unroll
-    for (int d = 0; d < 2 * kRing; ++d) {
-      const int n = n0 + d;
-      if (n < SL) {
-        const float2 c = cq[d % kRing];
-        if (n + kRing < SL) cq[d % kRing] = __ldg(co + (n + kRing) * CS);
-        mac_slot(n, c);
-      }
-    }
-    if (STG) cp_async_wait_group<0>();  // this thread's staged operands
-    {
-      // + w_N0 sum_N c_N, in FP64
-      const double cs = live ? (STG ? Cs[gi * FPB * R + it] : m.fcsum[f * R + r]) : 0.0;
-      double g[DIM];
-      if (STG) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) g[j] = fma(cs, Ws[(gi * FPB + fi) * DIM + j], ff_value(s[j], e[j]));
-      } else {
-        const int32_t id0 = __ldg(st + fi);
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) g[j] = fma(cs, __ldg(wd + j * ldw + id0), ff_value(s[j], e[j]));
-      }
-      if (MODE == kDfResidual || MODE == kDfFill) {
-        if (live && f >= m.nfi && f < m.nfid) {  // ghost node of a displacement face (prescribed data)
-          const int64_t fd = f - m.nfi;
-          const double cg = m.gco[fd * R + r];
-          const int q = r / DIM;
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) g[j] = fma(cg, ubq[(fd * Q + q) * DIM + j], g[j]);
-        }
-      }
-      const int64_t row = (f0 * R + it) * DIM;  // == (f * R + r) * DIM
-      if (MODE == kDfFill) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) m.gcache[row + j] = g[j];
-      }
-      if (MODE == kDfJv) {  // grad (u + eps v) = grad u + eps grad v
-        double* gr = Gs + (gi * FPB * R + it) * DIM;  // staged: this row of the cache
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) g[j] = fma(eps, g[j], STG ? gr[j] : m.gcache[row + j]);
-      }
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) Gs[(gi * FPB * R + it) * DIM + j] = g[j];
-    }
-    __syncthreads();  // the next group's gather overwrites the differences
-  }
-  // (2) law and traction at each Gauss point of the block's groups, one a thread
-  {
-    const int gi = it / (FPB * Q), rem = it % (FPB * Q), fj = rem / Q, q = rem % Q;
-    if (gi < ng) {
-      const int64_t grp = g0 + gi;
-      const int64_t fq = (grp / BPT) * kTile + (grp % BPT) * FPB + fj;
-      double t[DIM];
-      if (fq < m.nfid) {
-        double a[3];
-        const double* aq = STG ? As + ((gi * FPB + fj) * Q + q) * 3 : m.aq + (fq * Q + q) * 3;
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) a[k] = aq[k];
-        double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-        const double* gq = Gs + ((gi * FPB + fj) * R + q * DIM) * DIM;
-#pragma unroll
-        for (int i = 0; i < DIM; ++i)
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) G[i][j] = gq[i * DIM + j];
-        traction<DIM, LAW>(G, a, mt, t);
-      } else {
-#pragma unroll
-        for (int i = 0; i < DIM; ++i) t[i] = 0.0;
-      }
-      const int64_t o = (fq * Q + q) * DIM;
-      if (MODE == kDfFill) {
-#pragma unroll
-        for (int i = 0; i < DIM; ++i) m.tcache[o + i] = t[i];
-      }
-      if (MODE == kDfJv) {
-        const double* tc = STG ? Ts + ((gi * FPB + fj) * Q + q) * DIM : m.tcache + o;  // staged: this point
-#pragma unroll
-        for (int i = 0; i < DIM; ++i) t[i] -= tc[i];
-      }
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) Ts[((gi * FPB + fj) * Q + q) * DIM + i] = t[i];
+    for (int i = 0; i < DIM; ++i) {
+      if (MODE == kDfFill) m.tcache[tp * DIM + i * NP + pt] = t[i];
+      if (MODE == kDfJv) t[i] -= tu[i];
     }
   }
-  if (MODE == kDfFill) return;
-  __syncthreads();
-  // (3) quadrature over the face + alpha stabilisation
-  for (int t3 = it; t3 < ng * FPB * DIM; t3 += SH::THREADS) {
-    const int gi = t3 / (FPB * DIM), fj = (t3 / DIM) % FPB, i = t3 % DIM;
-    const int64_t grp = g0 + gi;
-    const int64_t ff = (grp / BPT) * kTile + (grp % BPT) * FPB + fj;
-    if (ff < m.nfid) {
-      double acc = 0.0;
-      for (int q = 0; q < Q; ++q) acc += Ts[((gi * FPB + fj) * Q + q) * DIM + i];
-      const int32_t sp = m.fstar[2 * ff], sn = m.fstar[2 * ff + 1];
-      const bool sym = sn < 0 && ff >= m.nfi + m.nfd;
-      const double up = ws[(int64_t)sp * DIM + i];
-      // beyond a displacement face: the prescribed value (the homogeneous and
-      // Jv modes differentiate it away)
-      const double other = sn >= 0 ? ws[(int64_t)sn * DIM + i]
-                           : sym   ? mirror_i<DIM>(ws + (int64_t)sp * DIM, m.nrm + 3 * ff, i)
-                           : MODE == kDfResidual ? ubf[(ff - m.nfi) * DIM + i]
-                                                 : 0.0;
-      // the stabilisation is linear: its difference at u + eps v and u is
-      // eps times its value at v
-      const double coef = mt.alpha * mt.kbar * m.fstab[ff] * (MODE == kDfJv ? eps : 1.0);
-      flux[ff * DIM + i] = fma(coef, other - up, acc);
-    }
-  }
-}
-
-// Packed variant for polyhedral faces of 8 fan slots (Q = 32 points, 96
-// rows a face).  The rows of the slots past a face's last corner carry no
-// area; rather than one thread for each row of FPB whole faces, a group here
-// is a run of consecutive faces of one tile whose rows with area fill the
-// block's kPackThreads threads (at most kPackMaxFaces faces; the host builds
-// the runs, DevMesh::pgrp).  Thread it of a group takes the group's it-th
-// row with area, and the gradients, tractions and staged operands are
-// indexed by packed row and packed point.  Everything else is k_flux_df's:
-// reference differences, register ring, staged operands, GPB groups one
-// after the other and then the law at all their points (at most
-// kPackThreads / 3 a group, one a thread), Gauss sums over the points with
-// area in the same order, stabilisation.  The fluxes equal k_flux_df's bit
-// for bit (the padded points add exact zeros there).
-template <int LAW, int MODE>
-__global__ void __launch_bounds__(kPackThreads, 2)
-    k_flux_df_pk(DevMesh m, Material mt, const float4* __restrict__ sw, const double* __restrict__ wd,
-                 const double* __restrict__ ws, const double* __restrict__ ubq,
-                 const double* __restrict__ ubf, const double* __restrict__ d_eps,
-                 double* __restrict__ flux) {
-  constexpr int DIM = 3, Q = 32, R = Q * DIM, PM = kPackMaxFaces, T = kPackThreads, GPB = 3;
-  constexpr int PTS = T / DIM;  // points with area of a group, at most
-  constexpr int kRing = 8;
-  constexpr int CS = kTile * R;  // coefficient stride between stencil slots
-  extern __shared__ __align__(16) double sm[];
-  const int S = m.S;
-  float4* us = reinterpret_cast<float4*>(sm);                         // [S][PM][DIM]
-  double* Gs = reinterpret_cast<double*>(us + (size_t)S * PM * DIM);  // [GPB][T][DIM]
-  double* Ts = Gs + GPB * T * DIM;                                    // [GPB][PTS][DIM]
-  double* As = Ts + GPB * PTS * DIM;                                  // [GPB][PTS][3]
-  double* Cs = As + GPB * PTS * 3;                                    // [T] row sums
-  double* Ws = Cs + T;                                                // [PM][DIM] reference values
-  int* rowp = reinterpret_cast<int*>(Ws + PM * DIM);                  // [GPB][PM + 1] row offsets
-  int* gf = rowp + GPB * (PM + 1);                                    // [GPB][2] first face, faces
-  const int64_t ldw = m.wst;
-  const int64_t g0 = (int64_t)blockIdx.x * GPB;
-  const int ng = (int)(m.npg - g0 < GPB ? m.npg - g0 : GPB);
-  const int it = threadIdx.x;
-  const double eps = MODE == kDfJv ? __ldg(d_eps) : 0.0;
-  if (it < GPB) {  // the block's groups and the prefix sums of their rows with area
-    int fa = 0, na = 0;
-    if (it < ng) {
-      fa = m.pgrp[2 * (g0 + it)];
-      na = m.pgrp[2 * (g0 + it) + 1];
-    }
-    gf[2 * it] = fa;
-    gf[2 * it + 1] = na;
-    int acc = 0;
-    rowp[it * (PM + 1)] = 0;
-    for (int k = 0; k < PM; ++k) {
-      if (k < na) acc += m.fql[fa + k] * DIM;
-      rowp[it * (PM + 1) + k + 1] = acc;
-    }
-  }
-  __syncthreads();
-  float2 cq[kRing];
-  for (int gi = 0; gi < ng; ++gi) {
-    const int f0 = gf[2 * gi], nf = gf[2 * gi + 1];
-    const int* rp = rowp + gi * (PM + 1);
-    const int64_t tile = f0 / kTile;
-    const int fb = f0 % kTile;
-    const int nrows = rp[nf];
-    int fi = 0;  // this thread's face in the group and its row there
-    while (fi + 1 < nf && rp[fi + 1] <= it) ++fi;
-    const bool live = it < nrows;
-    const int r = live ? it - rp[fi] : 0;
-    const int64_t f = f0 + fi;
-    const int32_t* __restrict__ st = m.fst + tile * (int64_t)S * kTile + fb;
-    const float2* __restrict__ co =
-        reinterpret_cast<const float2*>(m.fco) + tile * (int64_t)S * CS + (fb + fi) * R + r + CS;
-    const int SL = live ? S - 1 : 0;
+  if constexpr (MODE != kDfFill) {
 #pragma unroll
-    for (int d = 0; d < kRing; ++d) cq[d] = d < SL ? __ldg(co + d * CS) : make_float2(0.f, 0.f);
-    for (int t = it; t < S * nf; t += T) {
-      const int n = t / nf, fj = t % nf;
-      const int32_t id = __ldg(st + n * kTile + fj);
+    for (int i = 0; i < DIM; ++i) Ts[it * DIM + i] = t[i];
+    // quadrature over the face + alpha stabilisation, a thread a component of
+    // a face (SUMS of them where a face has fewer points than components);
+    // what does not depend on the tractions is loaded before they are ready
+    constexpr int SUMS = (FPB * DIM + T - 1) / T;
+    double up[SUMS], other[SUMS], coef[SUMS];
 #pragma unroll
-      for (int h = 0; h < DIM; ++h) cp_async16(us + (n * PM + fj) * DIM + h, sw + (int64_t)id * DIM + h);
-      if (n == 0) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) cp_async8(Ws + fj * DIM + j, wd + j * ldw + id);
+    for (int k = 0; k < SUMS; ++k) {
+      const int fs = (it + k * T) / DIM, i = (it + k * T) % DIM;
+      const int64_t ff = f0 + fs;
+      up[k] = other[k] = coef[k] = 0.0;
+      if (fs < nf) {
+        const int32_t sp = m.fstar[2 * ff], sn = m.fstar[2 * ff + 1];
+        const bool sym = sn < 0 && ff >= m.nfi + m.nfd;
+        up[k] = ws[(int64_t)sp * DIM + i];
+        // beyond a displacement face: the prescribed value (the homogeneous and
+        // Jv modes differentiate it away)
+        other[k] = sn >= 0 ? ws[(int64_t)sn * DIM + i]
+                   : sym   ? mirror_i<DIM>(ws + (int64_t)sp * DIM, m.nrm + 3 * ff, i)
+                   : MODE == kDfResidual ? ubf[(ff - m.nfi) * DIM + i]
+                                         : 0.0;
+        // the stabilisation is linear: its difference at u + eps v and u is
+        // eps times its value at v
+        coef[k] = mt.alpha * mt.kbar * m.fstab[ff] * (MODE == kDfJv ? __ldg(d_eps) : 1.0);
       }
-    }
-    cp_async_commit();
-    // second group: this thread's row sum and (Jv) cached gradient row, the
-    // group's area vectors and (Jv) cached tractions by packed point
-    if (live) {
-      cp_async8(Cs + it, m.fcsum + f * R + r);
-      if (MODE == kDfJv) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j)
-          cp_async8(Gs + (gi * T + it) * DIM + j, m.gcache + (f * R + r) * DIM + j);
-      }
-    }
-    if (it < nrows / DIM) {
-      const int p = it;
-      int fj = 0;
-      while (rp[fj + 1] <= p * DIM) ++fj;
-      const int q = p - rp[fj] / DIM;
-      const int64_t o = ((int64_t)(f0 + fj) * Q + q) * 3;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) cp_async8(As + (gi * PTS + p) * 3 + k, m.aq + o + k);
-      if (MODE == kDfJv) {
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) cp_async8(Ts + (gi * PTS + p) * DIM + k, m.tcache + o + k);
-      }
-    }
-    cp_async_commit();
-    cp_async_wait_group<1>();  // the gather
-    __syncthreads();
-    for (int t = it; t < (S - 1) * nf * DIM; t += T) {
-      const int n = 1 + t / (nf * DIM), k = t % (nf * DIM);
-      const int e = n * PM * DIM + k;  // k = fj * DIM + h
-      const float2 dv = diff3(us[e], us[k]);
-      us[e] = make_float4(dv.x, dv.y, 0.f, 0.f);
     }
     __syncthreads();
-    float s[DIM], e[DIM];
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) s[j] = e[j] = 0.f;
-    const float4* __restrict__ uf = us + PM * DIM + fi * DIM;  // slot 1 of the thread's face
-    auto mac_slot = [&](int n, float2 c) {
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        const float4 a = uf[n * PM * DIM + j];
-        ff_mac(c.x, c.y, a.x, a.y, s[j], e[j]);
-      }
-    };
-    int n0 = 0;
-    for (; n0 + 2 * kRing <= SL; n0 += kRing) {
-      const float2* cn = co + (n0 + kRing) * CS;
-#pragma unroll
-      for (int d = 0; d < kRing; ++d) {
-        const float2 c = cq[d];
-        cq[d] = __ldg(cn + d * CS);
-        mac_slot(n0 + d, c);
-      }
-    }
-#pragma unroll
-    for (int d = 0; d < 2 * kRing; ++d) {
-      const int n = n0 + d;
-      if (n < SL) {
-        const float2 c = cq[d % kRing];
-        if (n + kRing < SL) cq[d % kRing] = __ldg(co + (n + kRing) * CS);
-        mac_slot(n, c);
-      }
-    }
-    cp_async_wait_group<0>();
-    {
-      const double cs = live ? Cs[it] : 0.0;
-      double g[DIM];
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) g[j] = fma(cs, Ws[fi * DIM + j], ff_value(s[j], e[j]));
-      if (MODE == kDfResidual || MODE == kDfFill) {
-        if (live && f >= m.nfi && f < m.nfid) {  // ghost node of a displacement face
-          const int64_t fd = f - m.nfi;
-          const double cg = m.gco[fd * R + r];
-          const int q = r / DIM;
-#pragma unroll
-          for (int j = 0; j < DIM; ++j) g[j] = fma(cg, ubq[(fd * Q + q) * DIM + j], g[j]);
-        }
-      }
-      double* gr = Gs + (gi * T + it) * DIM;
-      if (MODE == kDfFill && live) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) m.gcache[(f * R + r) * DIM + j] = g[j];
-      }
-      if (MODE == kDfJv) {
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) g[j] = fma(eps, g[j], live ? gr[j] : 0.0);
-      }
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) gr[j] = g[j];
-    }
-    __syncthreads();  // the next group's gather overwrites the differences
-  }
-  // law at each point with area of the block's groups, one a thread
-  {
-    const int gi = it / PTS, p = it % PTS;
-    if (gi < ng) {
-      const int* rp = rowp + gi * (PM + 1);
-      const int nf = gf[2 * gi + 1];
-      if (p < rp[nf] / DIM) {
-        int fj = 0;
-        while (rp[fj + 1] <= p * DIM) ++fj;
-        const int q = p - rp[fj] / DIM;
-        const int64_t fq = gf[2 * gi] + fj;
-        double t[DIM];
-        if (fq < m.nfid) {
-          double a[3];
-#pragma unroll
-          for (int k = 0; k < DIM; ++k) a[k] = As[(gi * PTS + p) * 3 + k];
-          double G[3][3];
-          const double* gq = Gs + (gi * T + rp[fj] + q * DIM) * DIM;
-#pragma unroll
-          for (int i = 0; i < DIM; ++i)
-#pragma unroll
-            for (int j = 0; j < DIM; ++j) G[i][j] = gq[i * DIM + j];
-          traction<DIM, LAW>(G, a, mt, t);
-        } else {
-#pragma unroll
-          for (int i = 0; i < DIM; ++i) t[i] = 0.0;
-        }
-        double* tp = Ts + (gi * PTS + p) * DIM;
-        if (MODE == kDfFill) {
-#pragma unroll
-          for (int i = 0; i < DIM; ++i) m.tcache[(fq * Q + q) * DIM + i] = t[i];
-        }
-        if (MODE == kDfJv) {
-#pragma unroll
-          for (int i = 0; i < DIM; ++i) t[i] -= tp[i];
-        }
-#pragma unroll
-        for (int i = 0; i < DIM; ++i) tp[i] = t[i];
+    for (int k = 0; k < SUMS; ++k) {
+      const int fs = (it + k * T) / DIM, i = (it + k * T) % DIM;
+      const int64_t ff = f0 + fs;
+      if (fs < nf) {
+        const int p0 = PACK ? rowp[fs] : fs * Q, p1 = PACK ? rowp[fs + 1] : p0 + Q;
+        double acc = 0.0;
+        for (int p = p0; p < p1; ++p) acc += Ts[p * DIM + i];
+        flux[ff * DIM + i] = fma(coef[k], other[k] - up[k], acc);
       }
     }
   }
-  if (MODE == kDfFill) return;
-  __syncthreads();
-  // Gauss sums over each face's points with area + alpha stabilisation
-  for (int t3 = it; t3 < ng * PM * DIM; t3 += T) {
-    const int gi = t3 / (PM * DIM), fj = (t3 / DIM) % PM, i = t3 % DIM;
-    const int* rp = rowp + gi * (PM + 1);
-    if (fj >= gf[2 * gi + 1]) continue;
-    const int64_t ff = gf[2 * gi] + fj;
-    if (ff >= m.nfid) continue;
-    double acc = 0.0;
-    for (int p = rp[fj] / DIM; p < rp[fj + 1] / DIM; ++p) acc += Ts[(gi * PTS + p) * DIM + i];
-    const int32_t sp = m.fstar[2 * ff], sn = m.fstar[2 * ff + 1];
-    const bool sym = sn < 0 && ff >= m.nfi + m.nfd;
-    const double up = ws[(int64_t)sp * DIM + i];
-    const double other = sn >= 0 ? ws[(int64_t)sn * DIM + i]
-                         : sym   ? mirror_i<DIM>(ws + (int64_t)sp * DIM, m.nrm + 3 * ff, i)
-                         : MODE == kDfResidual ? ubf[(ff - m.nfi) * DIM + i]
-                                               : 0.0;
-    const double coef = mt.alpha * mt.kbar * m.fstab[ff] * (MODE == kDfJv ? eps : 1.0);
-    flux[ff * DIM + i] = fma(coef, other - up, acc);
-  }
-}
-
-static size_t df_pk_smem_bytes(int S) {
-  constexpr int PM = kPackMaxFaces, T = kPackThreads, GPB = 3, PTS = T / 3;
-  return (size_t)S * PM * 3 * 16 + sizeof(double) * (GPB * T * 3 + GPB * PTS * 3 * 2 + T + PM * 3) +
-         sizeof(int) * (GPB * (PM + 1) + GPB * 2);
-}
-
-template <int LAW, int MODE>
-static void launch_flux_df_pk(const DevMesh& m, const Material& mat, const float4* sw,
-                              const double* wd, const double* ws, const double* ubq,
-                              const double* ubf, const double* d_eps, double* flux, cudaStream_t st) {
-  if (m.npg == 0) return;
-  k_flux_df_pk<LAW, MODE><<<(unsigned)((m.npg + 2) / 3), kPackThreads, df_pk_smem_bytes(m.S), st>>>(
-      m, mat, sw, wd, ws, ubq, ubf, d_eps, flux);
 }
 
 // contracted linear form, homogeneous part at v: sum_N T_N v_N plus the
@@ -1599,24 +1523,28 @@ static void launch_ustar_df(const DevMesh& m, const float4* sw, const double* w,
                             cudaStream_t st) {
   by_faces_per_cell<DIM>(m, [&](auto nlf) {
     constexpr int NLF = decltype(nlf)::value;
-    k_ustar_df<DIM, NLF><<<(unsigned)m.nctile, 32 * NLF, 0, st>>>(m, sw, w, out);
+    using SH = UsShape<NLF>;
+    const int W = SH::split(m.S);
+    k_ustar_df<DIM, NLF><<<(unsigned)m.nctile, 32 * SH::NG * W, sizeof(float2) * W * NLF * DIM * 33, st>>>(
+        m, sw, w, out);
   });
 }
 
-template <int DIM, int LAW, int MODE, int QD>
+template <int DIM, int LAW, int MODE, int QD, bool PACK = false>
 static void launch_flux_df_q(const DevMesh& m, const Material& mat, const float4* sw,
                              const double* wd, const double* ws, const double* ubq,
                              const double* ubf, const double* d_eps, double* flux,
                              cudaStream_t st) {
-  using SH = DfShape<DIM, QD>;
-  const size_t smem = df_smem_bytes<DIM, QD>(m.S);
-  const int64_t groups = m.nftile * (kTile / SH::FPB);
-  k_flux_df<DIM, LAW, MODE, QD><<<(unsigned)((groups + SH::GPB - 1) / SH::GPB), SH::THREADS, smem,
-                                  st>>>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux);
+  using SH = DfShape<DIM, QD, PACK>;
+  const int64_t groups = PACK ? m.npg : (m.nfid + SH::FPB - 1) / SH::FPB;
+  if (groups == 0) return;
+  k_flux_df<DIM, LAW, MODE, QD, PACK><<<(unsigned)groups, SH::THREADS, df_smem_bytes<DIM, QD, PACK>(m.S), st>>>(
+      m, mat, sw, wd, ws, ubq, ubf, d_eps, flux);
 }
 
 // Gauss points per face: q^(d-1) for q = 1..4 in 2-D, 1..3 in 3-D; on
-// polyhedra 4 or 8 fan slots of q^2 points for q = 1, 2
+// polyhedra 4 or 8 fan slots of q^2 points for q = 1, 2 (8 slots of 4 points
+// always with their packed groups)
 template <int DIM, int LAW, int MODE>
 static void launch_flux_df(const DevMesh& m, const Material& mat, const float4* sw,
                            const double* wd, const double* ws, const double* ubq,
@@ -1634,9 +1562,7 @@ static void launch_flux_df(const DevMesh& m, const Material& mat, const float4* 
       case 4: return launch_flux_df_q<3, LAW, MODE, 4>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
       case 8: return launch_flux_df_q<3, LAW, MODE, 8>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
       case 16: return launch_flux_df_q<3, LAW, MODE, 16>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 32:
-        if (m.pgrp) return launch_flux_df_pk<LAW, MODE>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-        return launch_flux_df_q<3, LAW, MODE, 32>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
+      case 32: return launch_flux_df_q<3, LAW, MODE, 32, true>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
       default: return launch_flux_df_q<3, LAW, MODE, 9>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
     }
   }
@@ -1750,32 +1676,25 @@ void launch_jv_df(const DevMesh& m, const Material& mat, const double* v, const 
   }
 }
 
-// the face kernels' gathers exceed the default 48 KB of dynamic shared
+// the face kernels' differences exceed the default 48 KB of dynamic shared
 // memory for large stencils: raise the limit of every instantiation to what
 // kMaxS stencil cells need, once per process (set-up calls only, never
 // during stream capture)
-template <int DIM, int LAW, int MODE, int QD>
+template <int DIM, int LAW, int MODE, int QD, bool PACK>
 static void raise_smem(cudaError_t& e) {
   const cudaError_t r =
-      cudaFuncSetAttribute((const void*)k_flux_df<DIM, LAW, MODE, QD>,
+      cudaFuncSetAttribute((const void*)k_flux_df<DIM, LAW, MODE, QD, PACK>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)df_smem_bytes<DIM, QD>(kMaxS));
+                           (int)df_smem_bytes<DIM, QD, PACK>(kMaxS));
   if (r != cudaSuccess) e = r;
 }
-template <int LAW, int MODE>
-static void raise_smem_pk(cudaError_t& e) {
-  const cudaError_t r = cudaFuncSetAttribute((const void*)k_flux_df_pk<LAW, MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)df_pk_smem_bytes(kMaxS));
-  if (r != cudaSuccess) e = r;
-}
-template <int DIM, int QD>
+template <int DIM, int QD, bool PACK = false>
 static void raise_smem_all(cudaError_t& e) {
-  raise_smem<DIM, 0, kDfResidual, QD>(e);
-  raise_smem<DIM, 1, kDfResidual, QD>(e);
-  raise_smem<DIM, 0, kDfHomog, QD>(e);
-  raise_smem<DIM, 1, kDfFill, QD>(e);
-  raise_smem<DIM, 1, kDfJv, QD>(e);
+  raise_smem<DIM, 0, kDfResidual, QD, PACK>(e);
+  raise_smem<DIM, 1, kDfResidual, QD, PACK>(e);
+  raise_smem<DIM, 0, kDfHomog, QD, PACK>(e);
+  raise_smem<DIM, 1, kDfFill, QD, PACK>(e);
+  raise_smem<DIM, 1, kDfJv, QD, PACK>(e);
 }
 int setup_df_kernels() {
   static int rc = -1;
@@ -1790,12 +1709,7 @@ int setup_df_kernels() {
   raise_smem_all<3, 9>(e);
   raise_smem_all<3, 8>(e);
   raise_smem_all<3, 16>(e);
-  raise_smem_all<3, 32>(e);
-  raise_smem_pk<0, kDfResidual>(e);
-  raise_smem_pk<1, kDfResidual>(e);
-  raise_smem_pk<0, kDfHomog>(e);
-  raise_smem_pk<1, kDfFill>(e);
-  raise_smem_pk<1, kDfJv>(e);
+  raise_smem_all<3, 32, true>(e);
   rc = e == cudaSuccess ? 0 : (int)e;
   return rc;
 }
