@@ -932,8 +932,9 @@ int hofv_build_stencils(hofv_ctx* c) {
   TRY(dev_alloc(c, &c->d_scal, 256));
   HOFV_CUDA(c, cudaMemset(c->d_count, 0, sizeof(unsigned int) * 256));
   HOFV_CUDA(c, cudaMemset(c->d_scal, 0, sizeof(double) * 256));
-  TRY(dev_alloc(c, &c->d_cg64, 8 * nc * d));
-  TRY(dev_alloc(c, &c->d_cg32, 8 * nc * d));
+  // CG vectors: six of 2 or 4 elements a cell and two of d (k_cg_persist)
+  TRY(dev_alloc(c, &c->d_cg64, (6 * (d == 2 ? 2 : 4) + 2 * d) * nc));
+  TRY(dev_alloc(c, &c->d_cg32, (6 * (d == 2 ? 2 : 4) + 2 * d) * nc));
   HOFV_CUDA(c, cudaDeviceSynchronize());
   c->src_dirty = false;
   c->built = true;

@@ -207,12 +207,12 @@ struct hofv_ctx {
   double* d_aj_off = nullptr;       // [nc][nlf]
   float* d_aj_diag32 = nullptr;
   float* d_aj_off32 = nullptr;
-  unsigned int* d_bar = nullptr;    // grid barrier of the persistent CG: count, generation, error
+  unsigned int* d_bar = nullptr;    // grid barrier of the persistent CG: arrivals, blocks done, error
   double* d_aj_invd = nullptr;      // 1 / (-diag), FP64 and FP32
   float* d_aj_invd32 = nullptr;
-  // CG work vectors (sized dim*nc each)
-  double *d_cg64 = nullptr;         // 5 vectors FP64
-  float *d_cg32 = nullptr;          // 5 vectors FP32
+  // CG work vectors
+  double *d_cg64 = nullptr;         // r, w, s twice, x, p in FP64
+  float *d_cg32 = nullptr;          // the same in FP32
   // ---- Krylov ----
   int kry_m = 0;
   double* d_V = nullptr;            // [(m+1)][n]

@@ -322,132 +322,233 @@ __global__ void k_cg_finish(int64_t nc, const T* __restrict__ invd, const T* __r
 // per-block partial sums in the same fixed order.  The barrier's spin is
 // bounded: on time-out the kernel sets an error flag and returns, and the
 // host reports the error at its next synchronisation.
+//
+// An iteration touches a few hundred bytes a cell, all of it in L2 (or
+// registers), so its time is latency: the barrier, the reductions and the
+// gathers, 16 us an iteration on 32^2 quads and 24 us on 45^3 hexes when each
+// of these was a chain.  Hence:
+//  * One block of 1024 cells each, no more blocks than the cells need: 32^2
+//    quads run in one block and meet at its own barrier.
+//  * The 2 DIM inner products go together: interleaved shuffles, then one
+//    warp each for the sum over the warps and for the sum over the blocks.
+//  * Blocks wait on the arrivals themselves, without a sleep.
+//  * A cell's r, w and s are one vector load each for its neighbours; with a
+//    cell a thread (RES: at most 1024 cells a block and SM) its own values,
+//    its row of the matrix and x, p stay in registers.
+//  * alpha needs no quotient of the previous alpha: beta gamma / alpha_prev =
+//    beta^2 (delta - ...)_prev, gamma / beta = gamma_prev.
+// The sums keep their order (a warp's cells by shuffles in T, warps of 1024
+// cells in double, blocks in T), whatever the number of blocks.
 // ---------------------------------------------------------------------
-constexpr unsigned int kBarrierSpinLimit = 1u << 24;  // x ~64 ns sleeps: ~1 s
+constexpr unsigned int kBarrierSpinLimit = 1u << 22;  // polls of an L2 word, ~0.3 us each: ~1 s
 
 struct GridBarrier {
-  unsigned int* count;
-  unsigned int* gen;
+  unsigned int* count;  // arrivals since the launch began
+  unsigned int* done;   // blocks that finished (the last one clears both)
   int* err;
 };
 
-__device__ __forceinline__ bool grid_barrier(const GridBarrier& gb, unsigned int nblocks,
+// Arrive, and wait until `target` arrivals have been counted since the
+// launch began.  Returns false (the same for the whole block) when the wait
+// ran out or another block's did.
+__device__ __forceinline__ bool grid_barrier(const GridBarrier& gb, unsigned int target,
                                              unsigned int spin_limit = kBarrierSpinLimit) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned int* vgen = gb.gen;
-    volatile int* verr = gb.err;
-    const unsigned int g = *vgen;
     __threadfence();
+    atomicAdd(gb.count, 1u);
     int ok = 1;
-    if (atomicAdd(gb.count, 1u) == nblocks - 1) {
-      atomicExch(gb.count, 0u);
-      __threadfence();
-      atomicAdd(gb.gen, 1u);
-    } else {
-      unsigned int spins = 0;
-      while (*vgen == g) {
-        if (++spins > spin_limit || *verr) {
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
+    unsigned int spins = 0, now;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(gb.count) : "memory");
+      if (now >= target) break;
+      if (++spins > spin_limit || ((spins & 1023u) == 0 && *(volatile int*)gb.err)) {
+        ok = 0;
+        break;
       }
     }
     if (!ok) atomicExch(gb.err, 1);
     __threadfence();
-    s_ok = ok && !*verr;
+    s_ok = ok;
   }
   __syncthreads();
   return s_ok != 0;
 }
 
-constexpr int kPersistThreads = 1024;
+// end of a launch whose blocks met at grid_barrier: the last block to get
+// here clears the counters for the next one
+__device__ __forceinline__ void grid_barrier_leave(const GridBarrier& gb) {
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(gb.done, 1u) == gridDim.x - 1) {
+      atomicExch(gb.count, 0u);
+      atomicExch(gb.done, 0u);
+    }
+  }
+}
 
-template <typename T, int DIM, int NLF>
+// a product rounded by itself: where a sum of two products could be fused
+// either way, the order of rounding is written out
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// a cell's DIM values as one (DIM = 2, or float) or two vector accesses, past
+// L1: other SMs write them between barriers
+template <typename T, int DIM>
+struct CellVec {
+  static constexpr int N = DIM == 2 ? 2 : 4;  // elements a cell
+  static __device__ __forceinline__ void ld(const T* a, int64_t c, T (&v)[DIM]) {
+    if constexpr (sizeof(T) == 4 && DIM == 2) {
+      const float2 x = __ldcg(reinterpret_cast<const float2*>(a) + c);
+      v[0] = x.x, v[1] = x.y;
+    } else if constexpr (sizeof(T) == 4) {
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(a) + c);
+      v[0] = x.x, v[1] = x.y, v[2] = x.z;
+    } else {
+      const double2 x = __ldcg(reinterpret_cast<const double2*>(a + c * N));
+      v[0] = x.x, v[1] = x.y;
+      if constexpr (DIM == 3) v[2] = __ldcg(a + c * N + 2);
+    }
+  }
+  static __device__ __forceinline__ void st(T* a, int64_t c, const T (&v)[DIM]) {
+    if constexpr (sizeof(T) == 4 && DIM == 2) {
+      __stcg(reinterpret_cast<float2*>(a) + c, make_float2(v[0], v[1]));
+    } else if constexpr (sizeof(T) == 4) {
+      __stcg(reinterpret_cast<float4*>(a) + c, make_float4(v[0], v[1], v[2], 0.f));
+    } else {
+      __stcg(reinterpret_cast<double2*>(a + c * N), make_double2(v[0], v[1]));
+      if constexpr (DIM == 3) __stcg(a + c * N + 2, v[2]);
+    }
+  }
+};
+
+constexpr int kPersistThreads = 1024;
+constexpr int kPersistWarps = kPersistThreads / 32;
+
+// rwork: r, w, s of even and odd iterations, CellVec::N * nc elements each;
+// xwork: x and p, DIM * nc each (not RES)
+template <typename T, int DIM, int NLF, bool RES>
 __global__ void __launch_bounds__(kPersistThreads)
     k_cg_persist(int64_t nc, int iters, const double* __restrict__ v, double inv_kbar,
                  const T* __restrict__ diag, const T* __restrict__ invd,
-                 const int32_t* __restrict__ col, const T* __restrict__ off, T* x, T* p, T* r0,
-                 T* r1, T* w0, T* w1, T* s0, T* s1, double* part, GridBarrier gb,
-                 double* __restrict__ zout) {
-  __shared__ double sh[32];
-  __shared__ double s_sc[3 * DIM];  // gamma_prev, alpha, beta
-  __shared__ T s_ab[2 * DIM];       // alpha, beta in the vector precision
+                 const int32_t* __restrict__ col, const T* __restrict__ off, T* rwork, T* xwork,
+                 double* part, GridBarrier gb, double* __restrict__ zout) {
+  using CV = CellVec<T, DIM>;
+  constexpr int NS = 2 * DIM;              // inner products: gamma_j, delta_j interleaved
+  __shared__ double sh[NS][kPersistWarps];
+  __shared__ double s_sum[NS];
+  __shared__ T s_ab[2 * DIM];              // alpha, beta in the vector precision
   const unsigned int nb = gridDim.x;
-  T* r[2] = {r0, r1};
-  T* w[2] = {w0, w1};
-  T* s[2] = {s0, s1};
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t nv = CV::N * nc;
+  T* r[2] = {rwork, rwork + nv};
+  T* w[2] = {rwork + 2 * nv, rwork + 3 * nv};
+  T* s[2] = {rwork + 4 * nv, rwork + 5 * nv};
+  T* xa = xwork;
+  T* pa = xwork + (RES ? 0 : DIM * nc);
+  const int64_t c0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t cstep = (int64_t)gridDim.x * blockDim.x;
   T pg[DIM], pd[DIM];  // per-thread partials in the vector precision
+  // threads j < DIM: 1 / gamma, denominator and alpha of the last iteration
+  double inv_gp = 0.0, den_p = 0.0, alpha_p = 0.0;
+  // the thread's cell (RES)
+  T rD = 0, riD = 0, ro_r[DIM], wo_r[DIM], so_r[DIM], xr[DIM], pr[DIM];
   // ---- iteration 0: r0 = b, w0 = B D^-1 r0, x = p = 0, s_{-1} = 0
 #pragma unroll
-  for (int j = 0; j < DIM; ++j) pg[j] = pd[j] = (T)0;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-       c += (int64_t)gridDim.x * blockDim.x) {
+  for (int j = 0; j < DIM; ++j) {
+    pg[j] = pd[j] = (T)0;
+    ro_r[j] = wo_r[j] = so_r[j] = xr[j] = pr[j] = (T)0;
+  }
+  for (int64_t c = c0; c < nc; c += cstep) {
     const T D = -diag[c], iD = invd[c];
-    T u[DIM], ww[DIM];
+    T u[DIM], ww[DIM], bb[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
       const T b = (T)(-v[j * nc + c] * inv_kbar);
-      r[0][j * nc + c] = b;
-      u[j] = b * iD;
-      ww[j] = D * u[j];
-      x[j * nc + c] = (T)0;
-      p[j * nc + c] = (T)0;
-      s[1][j * nc + c] = (T)0;
-      pg[j] += b * u[j];
+      bb[j] = b;
+      u[j] = mul_rn(b, iD);
+      ww[j] = mul_rn(D, u[j]);
+      pg[j] = fma(b, u[j], pg[j]);
     }
 #pragma unroll
     for (int lf = 0; lf < NLF; ++lf) {
       const int32_t n2 = col[c * NLF + lf];
       if (n2 < 0) continue;
-      const T o = off[c * NLF + lf] * invd[n2];
+      const T o = mul_rn(off[c * NLF + lf], invd[n2]);
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) ww[j] -= o * (T)(-v[j * nc + n2] * inv_kbar);
+      for (int j = 0; j < DIM; ++j) ww[j] = fma(-o, (T)(-v[j * nc + n2] * inv_kbar), ww[j]);
     }
+    const T zero[DIM] = {};
+    CV::st(r[0], c, bb);
+    CV::st(w[0], c, ww);
+    CV::st(s[1], c, zero);
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
-      w[0][j * nc + c] = ww[j];
-      pd[j] += ww[j] * u[j];
+      pd[j] = fma(ww[j], u[j], pd[j]);
+      if (RES) {
+        ro_r[j] = bb[j];
+        wo_r[j] = ww[j];
+      } else {
+        xa[j * nc + c] = (T)0;
+        pa[j * nc + c] = (T)0;
+      }
     }
+    if (RES) rD = D, riD = iD;
   }
   for (int it = 0; it < iters; ++it) {
-    // partial sums of this block -> part[parity][2j(+1)][block]
-    double* pp = part + (int64_t)(it & 1) * 2 * DIM * nb;
+    // the block's sums: a warp's cells by shuffles in T, its warps in double
+    T q[NS];
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) {
-      const double a = block_sum_t(pg[j], sh);
-      const double b = block_sum_t(pd[j], sh);
-      if (threadIdx.x == 0) {
-        pp[(2 * j) * nb + blockIdx.x] = a;
-        pp[(2 * j + 1) * nb + blockIdx.x] = b;
-      }
-    }
-    if (!grid_barrier(gb, nb)) return;
-    // every block forms the same scalars in the same order
-    for (int j = 0; j < DIM; ++j) {
-      const double gamma = warp0_sum<T>(pp + (2 * j) * nb, nb);
-      const double delta = warp0_sum<T>(pp + (2 * j + 1) * nb, nb);
-      if (threadIdx.x == 0) {
-        double alpha, beta;
-        if (it == 0) {
-          beta = 0.0;
-          alpha = delta != 0.0 ? gamma / delta : 0.0;
-        } else {
-          const double gp = s_sc[j], ap = s_sc[DIM + j];
-          beta = gp != 0.0 ? gamma / gp : 0.0;
-          const double den = ap != 0.0 ? delta - beta * gamma / ap : 0.0;
-          alpha = den != 0.0 ? gamma / den : 0.0;
-        }
-        s_sc[j] = gamma;
-        s_sc[DIM + j] = alpha;
-        s_sc[2 * DIM + j] = beta;
-        s_ab[j] = (T)alpha;
-        s_ab[DIM + j] = (T)beta;
-      }
+    for (int j = 0; j < DIM; ++j) q[2 * j] = pg[j], q[2 * j + 1] = pd[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < NS; ++k) q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) sh[k][wid] = (double)q[k];
     }
     __syncthreads();
+    double* pp = part + (int64_t)(it & 1) * NS * nb;  // [2j (+1)][block], by parity
+    if (wid < NS) {
+      double t = sh[wid][lane];
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        if (nb == 1) s_sum[wid] = (double)(T)t;
+        else __stcg(pp + wid * nb + blockIdx.x, t);
+      }
+    }
+    if (nb == 1) {
+      __syncthreads();
+    } else {
+      if (!grid_barrier(gb, (unsigned int)(it + 1) * nb)) return;
+      if (wid < NS) {  // every block forms the same sums in the same order
+        T t = (T)0;
+#pragma unroll 5
+        for (unsigned int b = lane; b < nb; b += 32) t += (T)__ldcg(pp + wid * nb + b);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) s_sum[wid] = (double)t;
+      }
+      __syncthreads();
+    }
+    if (threadIdx.x < DIM) {
+      const int j = threadIdx.x;
+      const double gamma = s_sum[2 * j], delta = s_sum[2 * j + 1];
+      const double beta = gamma * inv_gp;  // 0 in the first iteration
+      const double den = it == 0 ? delta : alpha_p != 0.0 ? fma(-(beta * beta), den_p, delta) : 0.0;
+      const double alpha = den != 0.0 ? gamma / den : 0.0;
+      den_p = den;
+      alpha_p = alpha;
+      s_ab[j] = (T)alpha;
+      s_ab[DIM + j] = (T)beta;
+    }
+    __syncthreads();
+    // the next beta's divisor, while the other warps go on
+    if (threadIdx.x < DIM) {
+      const double gamma = s_sum[2 * threadIdx.x];
+      inv_gp = gamma != 0.0 ? 1.0 / gamma : 0.0;
+    }
     T alpha[DIM], beta[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
@@ -460,15 +561,22 @@ __global__ void __launch_bounds__(kPersistThreads)
     const T* so_ = s[i & 1];
     if (i == iters) {
       // last step: z = x + alpha (u + beta p), u = D^-1 r
-      for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-           c += (int64_t)gridDim.x * blockDim.x) {
-        const T iD = invd[c];
+      for (int64_t c = c0; c < nc; c += cstep) {
+        const T iD = RES ? riD : invd[c];
+        T ro[DIM];
+        if (RES) {
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) ro[j] = ro_r[j];
+        } else {
+          CV::ld(ro_, c, ro);
+        }
 #pragma unroll
         for (int j = 0; j < DIM; ++j) {
-          const int64_t k = j * nc + c;
-          zout[k] = (double)(x[k] + alpha[j] * (ro_[k] * iD + beta[j] * p[k]));
+          const T x = RES ? xr[j] : xa[j * nc + c], p = RES ? pr[j] : pa[j * nc + c];
+          zout[j * nc + c] = (double)fma(alpha[j], fma(ro[j], iD, mul_rn(beta[j], p)), x);
         }
       }
+      if (nb > 1) grid_barrier_leave(gb);
       return;
     }
     T* rn_ = r[i & 1];
@@ -476,48 +584,62 @@ __global__ void __launch_bounds__(kPersistThreads)
     T* sn_ = s[(i - 1) & 1];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) pg[j] = pd[j] = (T)0;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nc;
-         c += (int64_t)gridDim.x * blockDim.x) {
-      const T D = -diag[c], iD = invd[c];
-      T un[DIM], ww[DIM];
+    for (int64_t c = c0; c < nc; c += cstep) {
+      const T D = RES ? rD : -diag[c], iD = RES ? riD : invd[c];
+      T ro[DIM], wo[DIM], so[DIM], rn[DIM], s1[DIM], un[DIM], ww[DIM];
+      if (RES) {
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) ro[j] = ro_r[j], wo[j] = wo_r[j], so[j] = so_r[j];
+      } else {
+        CV::ld(ro_, c, ro);
+        CV::ld(wo_, c, wo);
+        CV::ld(so_, c, so);
+      }
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        const int64_t k = j * nc + c;
-        const T ro = ro_[k];
-        const T s1 = wo_[k] + beta[j] * so_[k];
-        const T rn = ro - alpha[j] * s1;
-        const T pv = ro * iD + beta[j] * p[k];
-        p[k] = pv;
-        x[k] += alpha[j] * pv;
-        sn_[k] = s1;
-        rn_[k] = rn;
-        un[j] = rn * iD;
-        ww[j] = D * un[j];
-        pg[j] += rn * un[j];
+        s1[j] = fma(beta[j], so[j], wo[j]);
+        rn[j] = fma(-alpha[j], s1[j], ro[j]);
+        const T pold = RES ? pr[j] : pa[j * nc + c];
+        const T pv = fma(ro[j], iD, mul_rn(beta[j], pold));
+        if (RES) {
+          pr[j] = pv;
+          xr[j] = fma(alpha[j], pv, xr[j]);
+        } else {
+          pa[j * nc + c] = pv;
+          xa[j * nc + c] = fma(alpha[j], pv, xa[j * nc + c]);
+        }
+        un[j] = mul_rn(rn[j], iD);
+        ww[j] = mul_rn(D, un[j]);
+        pg[j] = fma(rn[j], un[j], pg[j]);
       }
+      CV::st(sn_, c, s1);
+      CV::st(rn_, c, rn);
 #pragma unroll
       for (int lf = 0; lf < NLF; ++lf) {
         const int32_t n2 = col[c * NLF + lf];
         if (n2 < 0) continue;
-        const T o = off[c * NLF + lf] * invd[n2];
+        const T o = mul_rn(off[c * NLF + lf], invd[n2]);
+        T rb[DIM], wb[DIM], sb[DIM];
+        CV::ld(ro_, n2, rb);
+        CV::ld(wo_, n2, wb);
+        CV::ld(so_, n2, sb);
 #pragma unroll
-        for (int j = 0; j < DIM; ++j) {
-          const int64_t k = j * nc + n2;
-          ww[j] -= o * (ro_[k] - alpha[j] * (wo_[k] + beta[j] * so_[k]));
-        }
+        for (int j = 0; j < DIM; ++j)
+          ww[j] = fma(-o, fma(-alpha[j], fma(beta[j], sb[j], wb[j]), rb[j]), ww[j]);
       }
+      CV::st(wn_, c, ww);
 #pragma unroll
       for (int j = 0; j < DIM; ++j) {
-        wn_[j * nc + c] = ww[j];
-        pd[j] += ww[j] * un[j];
+        pd[j] = fma(ww[j], un[j], pd[j]);
+        if (RES) ro_r[j] = rn[j], wo_r[j] = ww[j], so_r[j] = s1[j];
       }
     }
   }
 }
 
-template <typename T, int DIM, int NLF>
-static bool cg_persist_run(hofv_ctx* c, const T* diag, const T* invd, const T* off, T* work,
-                           int iters, const double* v, double* zout) {
+template <typename T, int DIM, int NLF, bool RES>
+static bool cg_persist_launch(hofv_ctx* c, const T* diag, const T* invd, const T* off, T* work,
+                              int iters, const double* v, double* zout) {
   static int mb = -1;  // co-resident blocks of this instantiation, found once
   if (mb < 0) {
     int per_sm = 0, dev = 0, nsm = 0, coop = 0;
@@ -525,34 +647,48 @@ static bool cg_persist_run(hofv_ctx* c, const T* diag, const T* invd, const T* o
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (!coop ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_persist<T, DIM, NLF>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg_persist<T, DIM, NLF, RES>,
                                                       kPersistThreads, 0) != cudaSuccess)
       per_sm = 0;
-    mb = std::min(per_sm, 1) * nsm;
+    int blocks = std::min(per_sm, 1) * nsm;
     const char* env = getenv("HOFV_CG_PERSISTENT");
-    if (env && env[0] == '0') mb = 0;
+    if (env && env[0] == '0') blocks = 0;
+    mb = blocks;
   }
   if (mb <= 0 || !c->d_bar) return false;
-  const int64_t nc = c->nc, n = DIM * nc;
-  T* x = work;
-  T* p = work + n;
-  int64_t nc_ = nc;
+  int64_t nc = c->nc;
+  const int64_t need = (nc + kPersistThreads - 1) / kPersistThreads;
+  if (RES && need > mb) return false;
+  const unsigned int nb = (unsigned int)std::min<int64_t>(need, mb);
   int iters_ = std::max(iters, 1);
   double inv_kbar = 1.0 / c->mat.kbar;
-  T *r0 = work + 2 * n, *r1 = work + 3 * n, *w0 = work + 4 * n, *w1 = work + 5 * n;
-  T *s0 = work + 6 * n, *s1 = work + 7 * n;
+  T* rwork = work;
+  T* xwork = work + 6 * CellVec<T, DIM>::N * nc;
   double* part = c->d_red;
   GridBarrier gb{c->d_bar, c->d_bar + 1, reinterpret_cast<int*>(c->d_bar + 2)};
-  void* args[] = {&nc_, &iters_, (void*)&v, &inv_kbar, (void*)&diag, (void*)&invd,
-                  (void*)&c->d_aj_col, (void*)&off, &x, &p, &r0, &r1, &w0, &w1, &s0, &s1, &part,
-                  &gb, &zout};
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_cg_persist<T, DIM, NLF>, dim3(mb),
-                                                    dim3(kPersistThreads), args, 0, c->stream);
+  void* args[] = {&nc, &iters_, (void*)&v, &inv_kbar, (void*)&diag, (void*)&invd,
+                  (void*)&c->d_aj_col, (void*)&off, &rwork, &xwork, &part, &gb, &zout};
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_cg_persist<T, DIM, NLF, RES>,
+                                                    dim3(nb), dim3(kPersistThreads), args, 0,
+                                                    c->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return true;
+}
+
+template <typename T, int DIM, int NLF>
+static bool cg_persist_run(hofv_ctx* c, const T* diag, const T* invd, const T* off, T* work,
+                           int iters, const double* v, double* zout) {
+  // a cell a thread where one block an SM has threads for all cells (doubles
+  // do not fit the 64 registers of 1024 threads)
+  if constexpr (sizeof(T) == 4) {
+    if (c->nc <= (int64_t)kPersistThreads * c->sm_count &&
+        cg_persist_launch<T, DIM, NLF, true>(c, diag, invd, off, work, iters, v, zout))
+      return true;
+  }
+  return cg_persist_launch<T, DIM, NLF, false>(c, diag, invd, off, work, iters, v, zout);
 }
 
 template <typename T, int DIM, int NLF>
@@ -583,7 +719,7 @@ static void cg_run(hofv_ctx* c, const T* diag, const T* invd, const T* off, T* w
 // Two co-resident blocks wait at a barrier that expects one more arrival
 // than exists: the wait must run out and latch the error flag.
 __global__ void k_barrier_probe(GridBarrier gb, unsigned int spin_limit) {
-  grid_barrier(gb, gridDim.x + 1, spin_limit);
+  grid_barrier(gb, gridDim.x + 1, spin_limit);  // the count stays: the host clears it
 }
 
 int barrier_selftest(hofv_ctx* c, int* timed_out) {
