@@ -438,7 +438,7 @@ def step_section(args, wl, mesh, ctx, lay, u_ex, precision, rank, ws, peaks_dev,
     name = ("k_flux_df (double-float face gradients + law + quadrature, faces packed by "
             "their points with area)" if packed else
             "k_flux_df (double-float face gradients + law + quadrature)" if precision == "df64"
-            else "k_flux (FP64 face gradients + law + quadrature)")
+            else "k_flux (fixed-point face gradients + FP64 law + quadrature)")
     roofline = {
         "bound": "hbm", "achieved": jb / (jflux_ms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
         "frac": jb / (jflux_ms * 1e-3) / 1e9 / hbm,

@@ -84,6 +84,8 @@ DevMesh dev_mesh(const hofv_ctx* c) {
   m.tcache = c->d_tcache;
   m.kerr = c->d_bar ? c->d_bar + 3 : nullptr;
   m.fcsum = c->d_fcsum;
+  m.fexp = c->d_fexp;
+  m.cexp = c->d_cexp;
   return m;
 }
 
@@ -177,6 +179,7 @@ static void free_built(hofv_ctx* c) {
   c->d_ustar_v = c->d_vext = nullptr;
   c->d_gcache = c->d_tcache = nullptr;
   c->d_fcsum = nullptr;
+  c->d_fexp = c->d_cexp = nullptr;
   c->jv_u = c->jv_R = nullptr;
   c->jv_cur++;
   c->d_count = nullptr;
@@ -193,6 +196,15 @@ static void free_built(hofv_ctx* c) {
   c->built = false;
 }
 
+// row exponents of the coefficients, which the FP64 kernels scale by
+static int row_exponents(hofv_ctx* c) {
+  launch_row_exponents(c->d_fco, c->S, kTile * c->Q * c->dim, std::max<int64_t>(c->nftile, 1), c->d_fexp,
+                       c->stream);
+  launch_row_exponents(c->d_cex, c->S, kTile * c->nlf, c->nctile, c->d_cexp, c->stream);
+  HOFV_CUDA(c, cudaGetLastError());
+  return 0;
+}
+
 // rewrite the face and cell coefficient arrays as double-float pairs
 // (to_df = 1) or back to doubles (0), in place
 static int coef_format(hofv_ctx* c, int to_df) {
@@ -200,7 +212,10 @@ static int coef_format(hofv_ctx* c, int to_df) {
                      c->stream);
   launch_coef_format(c->d_cex, c->nctile * c->S, kTile, c->nlf, to_df, c->stream);
   c->prec = to_df ? HOFV_PREC_DF64 : HOFV_PREC_FP64;  // the arrays' format from here on
-  if (to_df) launch_row_sums(dev_mesh(c), c->d_fcsum, c->stream);
+  if (to_df)
+    launch_row_sums(dev_mesh(c), c->d_fcsum, c->stream);
+  else
+    TRY(row_exponents(c));
   HOFV_CUDA(c, cudaGetLastError());
   HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
   return 0;
@@ -777,10 +792,8 @@ int hofv_build_stencils(hofv_ctx* c) {
   TRY(dev_alloc(c, &c->d_cqx, nc * c->QC * 3));
   TRY(dev_alloc(c, &c->d_cqw, nc * c->QC));
   TRY(run_geometry(c));
-  // faces with more rows than one thread per (face, row) of a 32-face tile
-  // allows take the strided FP64 face kernel, whose shared memory is raised
-  if (kTile * c->Q * d > (d == 3 ? 864 : 256) &&
-      (d != 3 || c->Q > kPolyFaceMaxCorners * 4 || flux_wide_prepare() != 0))
+  // q <= 4 points an edge, q^2 <= 9 a face, or 8 fan slots of 4 points
+  if (kTile * c->Q * d > (d == 3 ? 864 : 256) && (d != 3 || c->Q > kPolyFaceMaxCorners * 4))
     return fail(c, HOFV_ENOTSUP, "too many face points for the face kernel");
   // reference length: power of two near the mean cell size (node bounding box)
   double vbox = 1.0;
@@ -922,10 +935,15 @@ int hofv_build_stencils(hofv_ctx* c) {
   TRY(dev_alloc(c, &c->d_fcsum, std::max<int64_t>(c->nftile, 1) * kTile * R));
   if (c->ng > 0) TRY(dev_alloc(c, &c->d_vext, (nc + c->ng) * d));
   {
-    const int e = setup_df_kernels();
+    const int e = setup_face_kernels();
     if (e != 0) return cuda_fail(c, (cudaError_t)e, "cudaFuncSetAttribute(face kernels)");
   }
-  if (c->prec == HOFV_PREC_DF64) TRY(coef_format(c, 1));
+  TRY(dev_alloc(c, &c->d_fexp, std::max<int64_t>(c->nftile, 1) * kTile * R));
+  TRY(dev_alloc(c, &c->d_cexp, c->nctile * kTile * nlf));
+  if (c->prec == HOFV_PREC_DF64)
+    TRY(coef_format(c, 1));
+  else
+    TRY(row_exponents(c));
   c->red_blocks = 4 * c->sm_count;
   TRY(dev_alloc(c, &c->d_red, (int64_t)c->red_blocks * 128));
   TRY(dev_alloc(c, &c->d_count, 256));
@@ -1980,7 +1998,10 @@ static int rebuild_from_stencils(hofv_ctx* c) {
     HOFV_CUDA(c, cudaMemsetAsync(c->d_cex + (c->nctile - 1) * ct, 0, sizeof(double) * ct, c->stream));
   }
   TRY(run_lsq(c));
-  if (c->prec == HOFV_PREC_DF64) TRY(coef_format(c, 1));
+  if (c->prec == HOFV_PREC_DF64)
+    TRY(coef_format(c, 1));
+  else
+    TRY(row_exponents(c));
   if (c->d_cmass) TRY(run_cell_mass(c));
   c->tco_valid = false;
   nej_release(c);

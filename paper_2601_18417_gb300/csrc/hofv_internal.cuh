@@ -95,6 +95,8 @@ struct DevMesh {
   double* gcache;         // [nftile][dim][dim][kTile * Q]
   double* tcache;         // [nftile][dim][kTile * Q]
   unsigned int* kerr;     // set to 1 by a face kernel whose bounded wait ran out
+  const uint16_t* fexp;   // [nftile][kTile][R] largest biased exponent of each gradient row
+  const uint16_t* cexp;   // [nctile][kTile][nlf] ... of each extrapolation row (HOFV_PREC_FP64)
   const double* fcsum;    // [nftile][dim][kTile * Q] sums over the stencil of the stored
                           // (double-float) gradient coefficients of each row
 };
@@ -185,6 +187,8 @@ struct hofv_ctx {
   float4* d_sv = nullptr;           // [nc + ng][split4] split Jv direction
   double* d_ustar_v = nullptr;      // [nc][nlf][dim]
   double* d_fcsum = nullptr;        // [nftile][dim][kTile * Q] row sums of the stored coefficients
+  uint16_t* d_fexp = nullptr;       // [nftile][kTile][R], FP64: row exponents of fco
+  uint16_t* d_cexp = nullptr;       // [nctile][kTile][nlf] ... of cex
   double* d_vext = nullptr;         // [dim][nc + ng]
   // neo-Hookean double-float Jv: face gradients and tractions at u, valid
   // for the state / residual pair (jv_u, jv_R) while jv_gen == jv_cur
@@ -281,7 +285,6 @@ DevMesh dev_mesh(const hofv_ctx* c);
 
 // ---- set-up kernels (setup.cu) ----
 int run_geometry(hofv_ctx* c);
-int flux_wide_prepare();
 int run_stencils(hofv_ctx* c, const std::vector<int64_t>& bucket_start,
                  const std::vector<int32_t>& bucket_items, const int nb[3], const double lo[3],
                  double bs);
@@ -324,9 +327,12 @@ void launch_coef_format(double* a, int64_t chunks, int np, int rows, int to_df, 
 // fcsum = sum over the stencil slots of the stored coefficients
 // (double-float pairs summed in FP64, in slot order)
 void launch_row_sums(const DevMesh& m, double* fcsum, cudaStream_t st);
-// raises the dynamic shared-memory limit of the double-float face kernels
+// out[tile][row] = the largest biased exponent over the S slots of each
+// coefficient row of a [tiles][S][cs], as the fixed-point contractions scale by
+void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_t* out, cudaStream_t st);
+// raises the dynamic shared-memory limit of the face and extrapolation kernels
 // (once per process, at set-up); 0 or a cudaError_t
-int setup_df_kernels();
+int setup_face_kernels();
 void launch_source(const hofv_ctx* c, cudaStream_t st);
 void launch_build_tco(const DevMesh& m, double mu, double lam, double* tco, cudaStream_t st);
 void launch_ghost_flux(const DevMesh& m, double mu, double lam, const double* ubq, double* gflux,

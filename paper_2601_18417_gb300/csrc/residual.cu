@@ -18,9 +18,10 @@
 //             stabilisation value), only when the mesh has symmetry faces
 //   k_cell_avg : inertia term of the BDF2 dynamics, only when enabled
 //
-// All arithmetic is FP64.  Every FP64 instruction of the gradient phase runs
-// with all 32 lanes busy: a tile's (face, row) pairs are laid out so that
-// consecutive threads own consecutive coefficient rows.
+// Operands and results are FP64; the contractions over the stencils are formed
+// in fixed point (more exact than FP64 FMAs, and not bound by their rate) or,
+// on request, in double-float arithmetic.  A tile's (face, row) pairs are laid
+// out so that consecutive threads own consecutive coefficient rows.
 #include <algorithm>
 #include <type_traits>
 
@@ -29,33 +30,258 @@
 namespace hofv {
 
 // ---------------------------------------------------------------------
+// Fixed-point contraction of FP64 coefficients with FP64 values (the
+// arithmetic of HOFV_PREC_FP64).
+//
+// GB300 issues 2 FP64 FMAs a clock and SM, a fraction of what one coefficient
+// a product needs at HBM speed, but many times that of 32 x 32 -> 64 bit
+// integer multiply-adds.  So a sum sum_N c_N u_N is formed exactly but for
+// the representation of its operands: the coefficients of a row in units of
+// 2^-56 of the row's largest binade (truncated, 56 bits), the values of a
+// stencil in units of 2^-55 of its largest (rounded, 55 bits), each as two
+// 28-bit limbs; the products of the high limbs and of the high with the low
+// ones are summed without rounding in 64 bits.  Left out are the products of
+// the low limbs (zero on average, the value's low limb being signed).  The
+// bounds |C1|, |C0| < 2^28, |U1|, |U0| <= 2^27 and kMaxS = 128 slots keep both
+// sums below 2^63.  A sum of FP64 FMAs rounds at 2^-53 of each partial sum, so
+// this is the more accurate of the two.
+//
+// Measured, FP64 FMAs -> this (us): k_flux 32^3 hexes p = 3 neo-Hookean 1424 ->
+// 666 (the FMAs alone bound it at 1140), 2 255^2 triangles p = 3 linear 107 ->
+// 88; k_ustar 32^3 hexes 102 -> 83, 512^2 quads 79 -> 64.
+//
+// Rows and stencils whose largest binade lies outside [kFxMin, kFxMax] (tiny,
+// huge, infinite or NaN values) are summed by FP64 FMAs.
+// ---------------------------------------------------------------------
+constexpr int kFxMin = 540, kFxMax = 1560;  // biased exponents: the scales stay normal numbers
+constexpr uint16_t kFxPlain = 0xffff;       // row exponent of a row to be summed by FMAs
+
+// largest biased exponent of each coefficient row of [tile][S][cs]
+__global__ void k_row_exponents(const double* __restrict__ a, int S, int cs, int64_t n,
+                                uint16_t* __restrict__ out) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (tile, row)
+  if (e >= n) return;
+  const double* __restrict__ p = a + e / cs * S * cs + e % cs;
+  int mx = 0;
+  bool zero = true;
+  for (int k = 0; k < S; ++k) {
+    const double v = p[(int64_t)k * cs];
+    zero &= v == 0.0;
+    mx = max(mx, (__double2hiint(v) >> 20) & 0x7ff);
+  }
+  out[e] = zero ? (uint16_t)kFxMin : mx < kFxMin || mx > kFxMax ? kFxPlain : (uint16_t)mx;
+}
+
+void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_t* out, cudaStream_t st) {
+  const int64_t n = tiles * cs;
+  if (n > 0) k_row_exponents<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, S, cs, n, out);
+}
+
+// |c| 2^(1078 - E) truncated, below 2^56, as 28-bit limbs (hi, lo) with c's sign
+__device__ __forceinline__ int2 fx_coef(double c, int E) {
+  const int h = __double2hiint(c);
+  const int sh = min(E - ((h >> 20) & 0x7ff), 63);  // 63 for zero: kFxMin
+  const uint64_t mant = (uint64_t)(uint32_t)((h & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(c);
+  const uint64_t v = (mant << 3) >> sh;
+  const int sg = (h >> 31) | 1;
+  return make_int2((int)(uint32_t)(v >> 28) * sg, (int)((uint32_t)v & 0xfffffffu) * sg);
+}
+
+// u 2^(1077 - E) rounded, at most 2^55, as 28-bit limbs (hi, lo), the low one
+// in [-2^27, 2^27)
+__device__ __forceinline__ int2 fx_value(int h, int l, int E) {
+  const int sh = min(E - ((h >> 20) & 0x7ff), 63);  // 63 for zero
+  const uint64_t mant = (uint64_t)(uint32_t)((h & 0xfffff) | 0x100000) << 32 | (uint32_t)l;
+  int64_t v = (int64_t)(((mant << 2) + ((1ull << sh) >> 1)) >> sh);
+  if (h < 0) v = -v;
+  const int64_t hi = (v + (1 << 27)) >> 28;
+  return make_int2((int)hi, (int)(v - (hi << 28)));
+}
+
+// hh 2^56 + x 2^28 in units of 2^(Ec - 1078 + Eu - 1077)
+__device__ __forceinline__ double fx_sum(int64_t hh, int64_t x, int Ec, int Eu) {
+  const int64_t t = hh + ((x + (1 << 27)) >> 28);
+  return (double)t * __hiloint2double((1023 + Ec + Eu - 2099) << 20, 0);
+}
+
+// The values at the stencils of `items` consecutive faces or cells (item0 the
+// first) as limbs in shared memory, ua[n * stride + k] components 0 and 1 and
+// ub component 2 of slot n of item k, and each item's exponents in ex (0 where
+// the item is to be summed by FMAs).  Called by the whole block.
+template <int DIM>
+__device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, const double* __restrict__ w,
+                                          int64_t ws, int S, int64_t item0, int items, int stride, int4* ua,
+                                          int2* ub, int* ex) {
+  constexpr int U = 4;
+  const int step = blockDim.x / stride, k = threadIdx.x % stride, s0 = threadIdx.x / stride;
+  const bool on = k < items && s0 < step;
+  const int64_t g = item0 + k;
+  const int32_t* __restrict__ st = sten + g / kTile * (int64_t)S * kTile + g % kTile;
+  for (int i = threadIdx.x; i < stride * DIM; i += blockDim.x) ex[i] = 0;
+  __syncthreads();
+  if (on) {
+    int mx[DIM];
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) mx[j] = 0;
+    for (int n0 = s0; n0 < S; n0 += U * step) {
+      int32_t id[U];  // the cells first: one wait for their list, one for their values
+#pragma unroll
+      for (int d = 0; d < U; ++d) id[d] = n0 + d * step < S ? __ldg(st + (n0 + d * step) * kTile) : 0;
+      double v[U][DIM];
+#pragma unroll
+      for (int d = 0; d < U; ++d)
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) v[d][j] = __ldg(w + j * ws + id[d]);
+#pragma unroll
+      for (int d = 0; d < U; ++d) {
+        const int n = n0 + d * step;
+        if (n >= S) break;
+        int h[DIM], l[DIM];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) {
+          h[j] = __double2hiint(v[d][j]);
+          l[j] = __double2loint(v[d][j]);
+          mx[j] = max(mx[j], (h[j] & 0x7fffffff) | (l[j] != 0));
+        }
+        ua[n * stride + k] = make_int4(h[0], l[0], h[1], l[1]);
+        if constexpr (DIM == 3) ub[n * stride + k] = make_int2(h[2], l[2]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) atomicMax(ex + k * DIM + j, mx[j]);
+  }
+  __syncthreads();
+  int E[DIM];
+  bool fx = true;
+  if (on) {
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+      const int key = ex[k * DIM + j];
+      E[j] = key == 0 ? kFxMin : key >> 20;  // all zero: any scale
+      fx &= E[j] >= kFxMin && E[j] <= kFxMax;
+    }
+  }
+  __syncthreads();
+  if (on) {
+    if (s0 == 0) {
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) ex[k * DIM + j] = fx ? E[j] : 0;
+    }
+    if (fx)
+      for (int n = s0; n < S; n += step) {  // a thread converts what it stored
+        const int4 a = ua[n * stride + k];
+        const int2 x = fx_value(a.x, a.y, E[0]), y = fx_value(a.z, a.w, E[1]);
+        ua[n * stride + k] = make_int4(x.x, x.y, y.x, y.y);
+        if constexpr (DIM == 3) {
+          const int2 b = ub[n * stride + k];
+          ub[n * stride + k] = fx_value(b.x, b.y, E[2]);
+        }
+      }
+  }
+  __syncthreads();
+}
+
+// acc[j] = sum over S slots of the row co (stride cs between slots) with the
+// values of item k; rowexp and ex[k] are their exponents.  `rows` slots are
+// requested ahead in registers.
+template <int DIM, int K>
+struct FxRow {
+  double c[K];
+  __device__ __forceinline__ void begin(const double* __restrict__ co, int64_t cs, int SL) {
+#pragma unroll
+    for (int d = 0; d < K; ++d) c[d] = d < SL ? __ldg(co + d * cs) : 0.0;
+  }
+  __device__ __forceinline__ void run(const double* __restrict__ co, int64_t cs, int SL, int E,
+                                      const int4* ua, const int2* ub, int stride, const int* ex,
+                                      double (&acc)[DIM]) {
+    int64_t hh[DIM], x[DIM];
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) hh[j] = x[j] = 0;
+    for (int n0 = 0; n0 < SL; n0 += K) {
+#pragma unroll
+      for (int d = 0; d < K; ++d) {
+        const int2 q = fx_coef(c[d], E);
+        if (n0 + d + K < SL) c[d] = __ldg(co + (n0 + d + K) * cs);
+        if (n0 + d < SL) {
+          const int4 a = ua[(n0 + d) * stride];
+          hh[0] += (int64_t)q.x * a.x;
+          x[0] += (int64_t)q.x * a.y;
+          x[0] += (int64_t)q.y * a.x;
+          hh[1] += (int64_t)q.x * a.z;
+          x[1] += (int64_t)q.x * a.w;
+          x[1] += (int64_t)q.y * a.z;
+          if constexpr (DIM == 3) {
+            const int2 b = ub[(n0 + d) * stride];
+            hh[2] += (int64_t)q.x * b.x;
+            x[2] += (int64_t)q.x * b.y;
+            x[2] += (int64_t)q.y * b.x;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) acc[j] = fx_sum(hh[j], x[j], E, ex[j]);
+  }
+};
+
+// the same sum by FP64 FMAs
+template <int DIM>
+__device__ __noinline__ void plain_row(const double* __restrict__ co, int64_t cs, int SL,
+                                       const int32_t* __restrict__ st, const double* __restrict__ w,
+                                       int64_t ws, double* acc) {
+  double s[DIM];
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) s[j] = 0.0;
+  for (int n = 0; n < SL; ++n) {
+    const int32_t id = __ldg(st + n * kTile);
+    const double c = __ldg(co + n * cs);
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) s[j] = fma(c, __ldg(w + j * ws + id), s[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) acc[j] = s[j];
+}
+
+// ---------------------------------------------------------------------
 // stabilisation extrapolation: one thread per (cell, local face)
 // ---------------------------------------------------------------------
 // NLF = faces per cell: 4 / 6 for quads / hexes, 3 / 4 for triangles / tetrahedra
+template <int DIM>
+constexpr int kUstarCells = DIM == 2 ? 32 : 16;  // cells a block: 3-D limbs fill shared memory sooner
+template <int DIM>
+static size_t fx_smem_bytes(int S, int items) {
+  return (size_t)S * items * DIM * sizeof(int2);
+}
+
 template <int DIM, int NLF>
-__global__ void __launch_bounds__(32 * NLF)
+__global__ void __launch_bounds__(kUstarCells<DIM> * NLF)
     k_ustar(DevMesh m, const double* __restrict__ w, double* __restrict__ ustar) {
-  const int64_t tile = blockIdx.x;
-  const int it = threadIdx.x;            // ci * NLF + lf
-  const int ci = it / NLF;
-  const int64_t cell = tile * kTile + ci;
-  const int32_t* __restrict__ st = m.cst + tile * m.S * kTile + ci;
-  const double* __restrict__ ex = m.cex + tile * (int64_t)m.S * kTile * NLF + it;
-  double acc[DIM];
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
+  constexpr int CPB = kUstarCells<DIM>;
+  extern __shared__ __align__(16) double sm[];
+  __shared__ int ex[CPB * DIM];
+  const int S = m.S;
+  int4* ua = reinterpret_cast<int4*>(sm);
+  int2* ub = reinterpret_cast<int2*>(ua + S * CPB);
+  const int64_t cell0 = (int64_t)blockIdx.x * CPB;
+  const int it = threadIdx.x, ci = it / NLF, lf = it % NLF;
+  const int64_t cell = cell0 + ci, tile = cell0 / kTile;
+  const bool on = cell < m.nc;
+  const int row = (int)(cell % kTile) * NLF + lf;
+  const double* __restrict__ co = m.cex + tile * (int64_t)S * kTile * NLF + row;
+  const int SL = on ? S : 0;
+  FxRow<DIM, 5> r;
+  r.begin(co, kTile * NLF, SL);
+  const int E = on ? m.cexp[tile * kTile * NLF + row] : kFxPlain;
   const int64_t ws = m.wst;  // stride of the state read
-#pragma unroll 4
-  for (int n = 0; n < m.S; ++n) {
-    const int32_t id = __ldg(st + n * kTile);
-    const double e = __ldg(ex + (int64_t)n * kTile * NLF);
+  fx_gather<DIM>(m.cst, w, ws, S, cell0, (int)min((int64_t)CPB, m.nc - cell0), CPB, ua, ub, ex);
+  if (!on) return;
+  double acc[DIM];
+  if (E != kFxPlain && ex[ci * DIM] != 0)
+    r.run(co, kTile * NLF, SL, E, ua + ci, ub + ci, CPB, ex + ci * DIM, acc);
+  else
+    plain_row<DIM>(co, kTile * NLF, SL, m.cst + tile * (int64_t)S * kTile + cell % kTile, w, ws, acc);
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) acc[j] = fma(e, __ldg(w + j * ws + id), acc[j]);
-  }
-  if (cell < m.nc) {
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) ustar[(cell * NLF + (it % NLF)) * DIM + j] = w[j * ws + cell] + acc[j];
-  }
+  for (int j = 0; j < DIM; ++j) ustar[(cell * NLF + lf) * DIM + j] = w[j * ws + cell] + acc[j];
 }
 
 // ---------------------------------------------------------------------
@@ -194,185 +420,102 @@ __device__ __forceinline__ void traction(const double (&G)[3][3], const double* 
 }
 
 // ---------------------------------------------------------------------
-// face fluxes, one tile of 32 faces per block, blockDim = 32 * R
+// face fluxes: FPB consecutive faces a block (a block may span two tiles),
+// one thread a (face, row) for the gradients, a (face, point) for the law and
+// a (face, component) for the quadrature
 // ---------------------------------------------------------------------
+constexpr int kFluxThreads = 384;
+// rows a block takes: as many whole faces, 32 at most, as give each row a
+// thread; R is at most 96 (8 fan slots of 2 x 2 points)
+static int flux_faces(int R) { return std::min(kTile, kFluxThreads / R); }
+static int flux_threads(int R) { return (flux_faces(R) * R + 31) / 32 * 32; }
+template <int DIM>
+static size_t flux_smem_bytes(int S, int R) {
+  const int F = flux_faces(R);
+  return fx_smem_bytes<DIM>(S, F) + sizeof(double) * F * (R * DIM + R);
+}
+
 template <int DIM, int LAW>
-__global__ void __launch_bounds__(DIM == 3 ? 864 : 256)
-    k_flux(DevMesh m, Material mt, const double* __restrict__ w, const double* __restrict__ ustar,
-           const double* __restrict__ ubq, const double* __restrict__ ubf,
-           double* __restrict__ flux) {
-  extern __shared__ double sm[];
+__global__ void __launch_bounds__(kFluxThreads, 3)
+    k_flux(DevMesh m, Material mt, int FPB, const double* __restrict__ w,
+           const double* __restrict__ ustar, const double* __restrict__ ubq,
+           const double* __restrict__ ubf, double* __restrict__ flux) {
+  extern __shared__ __align__(16) double sm[];
+  __shared__ int ex[kTile * DIM];
   const int R = m.R, Q = m.Q, S = m.S;
-  double* Gs = sm;                        // [32][R][DIM]
-  double* Ts = sm + kTile * R * DIM;      // [32][Q][DIM]
-  const int64_t tile = blockIdx.x;
+  int4* ua = reinterpret_cast<int4*>(sm);                                // [S][FPB] components 0, 1
+  int2* ub = reinterpret_cast<int2*>(ua + S * FPB);                      // [S][FPB] component 2
+  double* Gs = reinterpret_cast<double*>(ub + (DIM == 3 ? S * FPB : 0)); // [FPB][R][DIM]
+  double* Ts = Gs + FPB * R * DIM;                                       // [FPB][Q][DIM]
+  const int64_t f0 = (int64_t)blockIdx.x * FPB;
+  const int nf = (int)min((int64_t)FPB, m.nfid - f0);
   const int it = threadIdx.x;
   const int64_t nc = m.wst;  // stride of the state read
   // (1) gradient rows: thread (fi, r) accumulates sum_N c_{r,N} u_N
   {
     const int fi = it / R, r = it % R;
-    const int64_t f = tile * kTile + fi;
-    const int32_t* __restrict__ st = m.fst + tile * S * kTile + fi;
-    const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + it;
+    const int64_t f = f0 + fi, tile = f / kTile;
+    const int row = (int)(f % kTile) * R + r;
+    // rows of points without area (polyhedral fan slots past a face's last
+    // corner) are neither read nor formed
+    const bool live = fi < nf && (m.fql == nullptr || r < __ldg(m.fql + f) * DIM);
+    const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + row;
+    const int SL = live ? S : 0;
+    FxRow<DIM, 5> rw;
+    rw.begin(co, kTile * R, SL);
+    const int E = live ? m.fexp[tile * kTile * R + row] : kFxPlain;
+    fx_gather<DIM>(m.fst, w, nc, S, f0, nf, FPB, ua, ub, ex);
     double acc[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
-    // rows of points without area (polyhedral fan slots past a face's last
-    // corner) are neither read nor formed
-    const bool live = m.fql == nullptr || r < __ldg(m.fql + f) * DIM;
-#pragma unroll 4
-    for (int n = 0; n < (live ? S : 0); ++n) {
-      const int32_t id = __ldg(st + n * kTile);
-      const double c = __ldg(co + (int64_t)n * kTile * R);
+    if (live) {
+      if (E != kFxPlain && ex[fi * DIM] != 0)
+        rw.run(co, kTile * R, SL, E, ua + fi, ub + fi, FPB, ex + fi * DIM, acc);
+      else
+        plain_row<DIM>(co, kTile * R, SL, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc, acc);
+      if (f >= m.nfi && f < m.nfi + m.nfd) {  // ghost node of a displacement face
+        const int64_t fd = f - m.nfi;
+        const double cg = m.gco[fd * R + r];
+        const int q = r / DIM;
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) acc[j] = fma(c, __ldg(w + j * nc + id), acc[j]);
+        for (int j = 0; j < DIM; ++j) acc[j] = fma(cg, ubq[(fd * Q + q) * DIM + j], acc[j]);
+      }
     }
-    if (live && f >= m.nfi && f < m.nfid) {  // ghost node of a displacement face
-      const int64_t fd = f - m.nfi;
-      const double cg = m.gco[fd * R + r];
-      const int q = r / DIM;
+    if (fi < nf) {
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) acc[j] = fma(cg, ubq[(fd * Q + q) * DIM + j], acc[j]);
+      for (int j = 0; j < DIM; ++j) Gs[(fi * R + r) * DIM + j] = acc[j];
     }
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) Gs[(fi * R + r) * DIM + j] = acc[j];
   }
   __syncthreads();
   // (2) law and traction at each Gauss point
-  if (it < kTile * Q) {
+  if (it < nf * Q) {
     const int fi = it / Q, q = it % Q;
-    const int64_t f = tile * kTile + fi;
+    const int64_t f = f0 + fi;
     double t[DIM];
-    if (f < m.nfid) {
-      double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
 #pragma unroll
-      for (int i = 0; i < DIM; ++i)
+    for (int i = 0; i < DIM; ++i)
 #pragma unroll
-        for (int j = 0; j < DIM; ++j) G[i][j] = Gs[(fi * R + q * DIM + i) * DIM + j];
-      double a[3];
+      for (int j = 0; j < DIM; ++j) G[i][j] = Gs[(fi * R + q * DIM + i) * DIM + j];
+    double a[3];
 #pragma unroll
-      for (int k = 0; k < DIM; ++k) a[k] = m.aq[(f * Q + q) * 3 + k];
-      traction<DIM, LAW>(G, a, mt, t);
-    } else {
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) t[i] = 0.0;
-    }
+    for (int k = 0; k < DIM; ++k) a[k] = m.aq[(f * Q + q) * 3 + k];
+    traction<DIM, LAW>(G, a, mt, t);
 #pragma unroll
     for (int i = 0; i < DIM; ++i) Ts[(fi * Q + q) * DIM + i] = t[i];
   }
   __syncthreads();
   // (3) quadrature over the face + alpha stabilisation
-  if (it < kTile * DIM) {
+  if (it < nf * DIM) {
     const int fi = it / DIM, i = it % DIM;
-    const int64_t f = tile * kTile + fi;
-    if (f < m.nfid) {
-      double s = 0.0;
-      for (int q = 0; q < Q; ++q) s += Ts[(fi * Q + q) * DIM + i];
-      const int32_t sp = m.fstar[2 * f], sn = m.fstar[2 * f + 1];
-      const double other = sn >= 0 ? ustar[(int64_t)sn * DIM + i] : ubf[(f - m.nfi) * DIM + i];
-      const double coef = mt.alpha * mt.kbar * m.fstab[f];
-      flux[f * DIM + i] = fma(coef, other - ustar[(int64_t)sp * DIM + i], s);
-    }
+    const int64_t f = f0 + fi;
+    double s = 0.0;
+    for (int q = 0; q < Q; ++q) s += Ts[(fi * Q + q) * DIM + i];
+    const int32_t sp = m.fstar[2 * f], sn = m.fstar[2 * f + 1];
+    const double other = sn >= 0 ? ustar[(int64_t)sn * DIM + i] : ubf[(f - m.nfi) * DIM + i];
+    const double coef = mt.alpha * mt.kbar * m.fstab[f];
+    flux[f * DIM + i] = fma(coef, other - ustar[(int64_t)sp * DIM + i], s);
   }
-}
-
-// ---------------------------------------------------------------------
-// the same three phases for faces with more points than one thread per
-// (face, row) of a 32-face tile allows (polyhedral faces: up to 8 fan
-// triangles of q^2 points, R up to 96): kWideThreads threads walk the rows
-// and points of the tile in strides
-// ---------------------------------------------------------------------
-constexpr int kWideThreads = 512;
-
-template <int DIM, int LAW>
-__global__ void __launch_bounds__(kWideThreads)
-    k_flux_wide(DevMesh m, Material mt, const double* __restrict__ w,
-                const double* __restrict__ ustar, const double* __restrict__ ubq,
-                const double* __restrict__ ubf, double* __restrict__ flux) {
-  extern __shared__ double sm[];
-  const int R = m.R, Q = m.Q, S = m.S;
-  double* Gs = sm;                        // [32][R][DIM]
-  double* Ts = sm + kTile * R * DIM;      // [32][Q][DIM]
-  const int64_t tile = blockIdx.x;
-  const int64_t nc = m.wst;
-  for (int it = threadIdx.x; it < kTile * R; it += blockDim.x) {
-    const int fi = it / R, r = it % R;
-    const int64_t f = tile * kTile + fi;
-    const int32_t* __restrict__ st = m.fst + tile * S * kTile + fi;
-    const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + it;
-    double acc[DIM];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
-    // rows of points without area (polyhedral fan slots past a face's last
-    // corner) are neither read nor formed
-    const bool live = m.fql == nullptr || r < __ldg(m.fql + f) * DIM;
-#pragma unroll 4
-    for (int n = 0; n < (live ? S : 0); ++n) {
-      const int32_t id = __ldg(st + n * kTile);
-      const double c = __ldg(co + (int64_t)n * kTile * R);
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) acc[j] = fma(c, __ldg(w + j * nc + id), acc[j]);
-    }
-    if (live && f >= m.nfi && f < m.nfid) {
-      const int64_t fd = f - m.nfi;
-      const double cg = m.gco[fd * R + r];
-      const int q = r / DIM;
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) acc[j] = fma(cg, ubq[(fd * Q + q) * DIM + j], acc[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) Gs[(fi * R + r) * DIM + j] = acc[j];
-  }
-  __syncthreads();
-  for (int it = threadIdx.x; it < kTile * Q; it += blockDim.x) {
-    const int fi = it / Q, q = it % Q;
-    const int64_t f = tile * kTile + fi;
-    double t[DIM];
-    if (f < m.nfid) {
-      double G[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-#pragma unroll
-      for (int i = 0; i < DIM; ++i)
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) G[i][j] = Gs[(fi * R + q * DIM + i) * DIM + j];
-      double a[3];
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) a[k] = m.aq[(f * Q + q) * 3 + k];
-      traction<DIM, LAW>(G, a, mt, t);
-    } else {
-#pragma unroll
-      for (int i = 0; i < DIM; ++i) t[i] = 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < DIM; ++i) Ts[(fi * Q + q) * DIM + i] = t[i];
-  }
-  __syncthreads();
-  for (int it = threadIdx.x; it < kTile * DIM; it += blockDim.x) {
-    const int fi = it / DIM, i = it % DIM;
-    const int64_t f = tile * kTile + fi;
-    if (f < m.nfid) {
-      double s = 0.0;
-      for (int q = 0; q < Q; ++q) s += Ts[(fi * Q + q) * DIM + i];
-      const int32_t sp = m.fstar[2 * f], sn = m.fstar[2 * f + 1];
-      const double other = sn >= 0 ? ustar[(int64_t)sn * DIM + i] : ubf[(f - m.nfi) * DIM + i];
-      const double coef = mt.alpha * mt.kbar * m.fstab[f];
-      flux[f * DIM + i] = fma(coef, other - ustar[(int64_t)sp * DIM + i], s);
-    }
-  }
-}
-
-// dynamic shared memory of k_flux_wide beyond the default 48 KB, raised to
-// what the largest polyhedral face (8 fan slots of 2 x 2 points) needs, so
-// that contexts of different point counts never lower it for one another;
-// set for both laws before the first launch or capture
-int flux_wide_prepare() {
-  constexpr int kMaxWideQ = kPolyFaceMaxCorners * 4;
-  const int smem = (int)(sizeof(double) * kTile * (kMaxWideQ * 3 * 3 + kMaxWideQ * 3));
-  if (cudaFuncSetAttribute(k_flux_wide<3, HOFV_LAW_LINEAR>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_flux_wide<3, HOFV_LAW_NEOHOOKEAN>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return -1;
-  return 0;
 }
 
 // ---------------------------------------------------------------------
@@ -487,7 +630,9 @@ static void residual_impl(const DevMesh& m, const Material& mat, const double* w
   }
   by_faces_per_cell<DIM>(m, [&](auto nlf) {
     constexpr int NLF = decltype(nlf)::value;
-    k_ustar<DIM, NLF><<<(unsigned)m.nctile, 32 * NLF, 0, st>>>(m, w, ustar);
+    constexpr int CPB = kUstarCells<DIM>;
+    k_ustar<DIM, NLF><<<(unsigned)((m.nc + CPB - 1) / CPB), CPB * NLF, fx_smem_bytes<DIM>(m.S, CPB), st>>>(
+        m, w, ustar);
   });
   if (m.nfy > 0) k_sym_other<DIM><<<(unsigned)((m.nfy + 127) / 128), 128, 0, st>>>(m, ustar);
   if (ev) cudaEventRecord(ev[1], st);
@@ -496,14 +641,9 @@ static void residual_impl(const DevMesh& m, const Material& mat, const double* w
       k_tflux<DIM><<<(unsigned)m.nftile, 32 * DIM, 0, st>>>(m, m.tco, mat.alpha * mat.kbar, w,
                                                             ustar, ubf, flux);
     } else {
-      const size_t smem = sizeof(double) * kTile * (m.R * DIM + m.Q * DIM);
-      if (kTile * m.R <= (DIM == 3 ? 864 : 256)) {
-        k_flux<DIM, LAW><<<(unsigned)m.nftile, kTile * m.R, smem, st>>>(m, mat, w, ustar, ubq,
-                                                                        ubf, flux);
-      } else if constexpr (DIM == 3) {  // set-up admits no wider 2-D face
-        k_flux_wide<DIM, LAW><<<(unsigned)m.nftile, kWideThreads, smem, st>>>(m, mat, w, ustar,
-                                                                              ubq, ubf, flux);
-      }
+      const int fpb = flux_faces(m.R);
+      k_flux<DIM, LAW><<<(unsigned)((m.nfid + fpb - 1) / fpb), flux_threads(m.R),
+                         flux_smem_bytes<DIM>(m.S, m.R), st>>>(m, mat, fpb, w, ustar, ubq, ubf, flux);
     }
   }
   if (ev) cudaEventRecord(ev[2], st);
@@ -1676,8 +1816,8 @@ void launch_jv_df(const DevMesh& m, const Material& mat, const double* v, const 
   }
 }
 
-// the face kernels' differences exceed the default 48 KB of dynamic shared
-// memory for large stencils: raise the limit of every instantiation to what
+// the face kernels' differences and limbs exceed the default 48 KB of dynamic
+// shared memory for large stencils: raise the limit of every instantiation to what
 // kMaxS stencil cells need, once per process (set-up calls only, never
 // during stream capture)
 template <int DIM, int LAW, int MODE, int QD, bool PACK>
@@ -1696,10 +1836,34 @@ static void raise_smem_all(cudaError_t& e) {
   raise_smem<DIM, 1, kDfFill, QD, PACK>(e);
   raise_smem<DIM, 1, kDfJv, QD, PACK>(e);
 }
-int setup_df_kernels() {
+template <typename K>
+static void raise_smem_fx(cudaError_t& e, K* kernel, size_t bytes) {
+  const cudaError_t r =
+      cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (r != cudaSuccess) e = r;
+}
+template <int DIM, int NLF>
+static void raise_smem_ustar(cudaError_t& e) {
+  raise_smem_fx(e, k_ustar<DIM, NLF>, fx_smem_bytes<DIM>(kMaxS, kUstarCells<DIM>));
+}
+template <int DIM>
+static void raise_smem_flux(cudaError_t& e) {
+  // 32 faces of at most 12 rows need the most
+  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_LINEAR>, flux_smem_bytes<DIM>(kMaxS, kFluxThreads / kTile));
+  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_NEOHOOKEAN>, flux_smem_bytes<DIM>(kMaxS, kFluxThreads / kTile));
+}
+int setup_face_kernels() {
   static int rc = -1;
   if (rc >= 0) return rc;
   cudaError_t e = cudaSuccess;
+  raise_smem_ustar<2, 3>(e);
+  raise_smem_ustar<2, 4>(e);
+  raise_smem_ustar<2, kPolyMaxSides>(e);
+  raise_smem_ustar<3, 4>(e);
+  raise_smem_ustar<3, 6>(e);
+  raise_smem_ustar<3, kPolyhedronMaxFaces>(e);
+  raise_smem_flux<2>(e);
+  raise_smem_flux<3>(e);
   raise_smem_all<2, 1>(e);
   raise_smem_all<2, 2>(e);
   raise_smem_all<2, 3>(e);
