@@ -81,7 +81,7 @@ def kernel_hash():
     import re
     text = open(os.path.join(ROOT, "paper_2601_18417_gb300", "csrc", "residual.cu")).read()
     parts = []
-    for lo, hi in (("// laws: traction t = T a", "// face fluxes, one tile of 32 faces"),
+    for lo, hi in (("// laws: traction t = T a", "// face fluxes: FPB consecutive faces"),
                    ("// Face fluxes, double-float gradient rows.",
                     "// contracted linear form, homogeneous part at v")):
         a, b = text.find(lo), text.find(hi)

@@ -46,9 +46,15 @@ namespace hofv {
 // sums below 2^63.  A sum of FP64 FMAs rounds at 2^-53 of each partial sum, so
 // this is the more accurate of the two.
 //
-// Measured, FP64 FMAs -> this (us): k_flux 32^3 hexes p = 3 neo-Hookean 1424 ->
-// 666 (the FMAs alone bound it at 1140), 2 255^2 triangles p = 3 linear 107 ->
-// 88; k_ustar 32^3 hexes 102 -> 83, 512^2 quads 79 -> 64.
+// What bounds it: integer issue.  A coefficient takes about 15 instructions to
+// split and, for three components, nine multiply-adds at 32 a clock and SM (209
+// of the 467 us on 32^3 hexes; the bytes take 257).  Measured, FP64 FMAs -> this
+// (us): k_flux 32^3 hexes p = 3 neo-Hookean 1427 -> 467 (the FMAs alone bound it
+// at 1140), 40^3 p = 2 1074 -> 353, 2 255^2 triangles 107 -> 68, 20-layer prisms
+// 1107 -> 397, 6 17^3 tetrahedra 268 -> 116; k_ustar 32^3 hexes 102 -> 59, 512^2
+// quads 78 -> 57.  Strides known to the compiler and a loop without range checks
+// gave 666 -> 497 of that, the significand taken from the top of its word 478.
+// Not kept: every 5th slot by FP64 FMAs beside the others (515), two of five (682).
 //
 // Rows and stencils whose largest binade lies outside [kFxMin, kFxMax] (tiny,
 // huge, infinite or NaN values) are summed by FP64 FMAs.
@@ -80,11 +86,15 @@ void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_
 // |c| 2^(1078 - E) truncated, below 2^56, as 28-bit limbs (hi, lo) with c's sign
 __device__ __forceinline__ int2 fx_coef(double c, int E) {
   const int h = __double2hiint(c);
-  const int sh = min(E - ((h >> 20) & 0x7ff), 63);  // 63 for zero: kFxMin
-  const uint64_t mant = (uint64_t)(uint32_t)((h & 0xfffff) | 0x100000) << 32 | (uint32_t)__double2loint(c);
-  const uint64_t v = (mant << 3) >> sh;
-  const int sg = (h >> 31) | 1;
-  return make_int2((int)(uint32_t)(v >> 28) * sg, (int)((uint32_t)v & 0xfffffffu) * sg);
+  const uint32_t l = (uint32_t)__double2loint(c);
+  const int sh = min(E - ((h >> 20) & 0x7ff), 55);  // 55 for zero: kFxMin
+  // the significand at the top of 64 bits
+  const uint32_t mh = __funnelshift_l(l, (uint32_t)h, 11) | 0x80000000u;
+  const uint64_t m = (uint64_t)mh << 32 | (l << 11);
+  uint32_t hi;  // a shift by 32 and more gives zero
+  asm("shr.u32 %0, %1, %2;" : "=r"(hi) : "r"(mh), "r"(sh + 4));
+  const int lo = (int)((uint32_t)(m >> (sh + 8)) & 0xfffffffu);
+  return h < 0 ? make_int2(-(int)hi, -lo) : make_int2((int)hi, lo);
 }
 
 // u 2^(1077 - E) rounded, at most 2^55, as 28-bit limbs (hi, lo), the low one
@@ -92,32 +102,42 @@ __device__ __forceinline__ int2 fx_coef(double c, int E) {
 __device__ __forceinline__ int2 fx_value(int h, int l, int E) {
   const int sh = min(E - ((h >> 20) & 0x7ff), 63);  // 63 for zero
   const uint64_t mant = (uint64_t)(uint32_t)((h & 0xfffff) | 0x100000) << 32 | (uint32_t)l;
-  int64_t v = (int64_t)(((mant << 2) + ((1ull << sh) >> 1)) >> sh);
+  int64_t v = (int64_t)((((mant << 3) >> sh) + 1) >> 1);
   if (h < 0) v = -v;
   const int64_t hi = (v + (1 << 27)) >> 28;
-  return make_int2((int)hi, (int)(v - (hi << 28)));
+  return make_int2((int)hi, (int)((uint32_t)v - ((uint32_t)hi << 28)));
 }
 
-// hh 2^56 + x 2^28 in units of 2^(Ec - 1078 + Eu - 1077)
-__device__ __forceinline__ double fx_sum(int64_t hh, int64_t x, int Ec, int Eu) {
-  const int64_t t = hh + ((x + (1 << 27)) >> 28);
+// t in units of 2^56 2^(Ec - 1078 + Eu - 1077)
+__device__ __forceinline__ double fx_scale(int64_t t, int Ec, int Eu) {
   return (double)t * __hiloint2double((1023 + Ec + Eu - 2099) << 20, 0);
 }
 
+// sums of products of one component: the high limbs' (2^56) and the mixed (2^28)
+struct FxSum {
+  int64_t hh = 0, x = 0;
+  __device__ __forceinline__ void mac(int2 q, int uh, int ul) {
+    hh += (int64_t)q.x * uh;
+    x += (int64_t)q.x * ul;
+    x += (int64_t)q.y * uh;
+  }
+  __device__ __forceinline__ int64_t total() const { return hh + ((x + (1 << 27)) >> 28); }
+};
+
 // The values at the stencils of `items` consecutive faces or cells (item0 the
-// first) as limbs in shared memory, ua[n * stride + k] components 0 and 1 and
+// first) as limbs in shared memory, ua[n * STRIDE + k] components 0 and 1 and
 // ub component 2 of slot n of item k, and each item's exponents in ex (0 where
 // the item is to be summed by FMAs).  Called by the whole block.
-template <int DIM>
+template <int DIM, int THREADS, int STRIDE>
 __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, const double* __restrict__ w,
-                                          int64_t ws, int S, int64_t item0, int items, int stride, int4* ua,
-                                          int2* ub, int* ex) {
-  constexpr int U = 4;
-  const int step = blockDim.x / stride, k = threadIdx.x % stride, s0 = threadIdx.x / stride;
+                                          int64_t ws, int S, int64_t item0, int items, int4* ua, int2* ub,
+                                          int* ex) {
+  constexpr int U = 4, stride = STRIDE, step = THREADS / STRIDE;
+  const int k = threadIdx.x % stride, s0 = threadIdx.x / stride;
   const bool on = k < items && s0 < step;
   const int64_t g = item0 + k;
   const int32_t* __restrict__ st = sten + g / kTile * (int64_t)S * kTile + g % kTile;
-  for (int i = threadIdx.x; i < stride * DIM; i += blockDim.x) ex[i] = 0;
+  for (int i = threadIdx.x; i < stride * DIM; i += THREADS) ex[i] = 0;
   __syncthreads();
   if (on) {
     int mx[DIM];
@@ -181,46 +201,55 @@ __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, cons
   __syncthreads();
 }
 
-// acc[j] = sum over S slots of the row co (stride cs between slots) with the
-// values of item k; rowexp and ex[k] are their exponents.  `rows` slots are
-// requested ahead in registers.
-template <int DIM, int K>
+// Streams the S coefficients of the row co (CS between slots) as limbs to
+// mac(limbs, n0, d), slot n0 + d; E is the row's exponent.  K slots are requested
+// ahead in registers (begin, before the values are ready).
+template <int K, int CS>
 struct FxRow {
   double c[K];
-  __device__ __forceinline__ void begin(const double* __restrict__ co, int64_t cs, int SL) {
+  __device__ __forceinline__ void begin(const double* __restrict__ co, int S) {
 #pragma unroll
-    for (int d = 0; d < K; ++d) c[d] = d < SL ? __ldg(co + d * cs) : 0.0;
+    for (int d = 0; d < K; ++d) c[d] = d < S ? __ldg(co + d * CS) : 0.0;
   }
-  __device__ __forceinline__ void run(const double* __restrict__ co, int64_t cs, int SL, int E,
-                                      const int4* ua, const int2* ub, int stride, const int* ex,
-                                      double (&acc)[DIM]) {
-    int64_t hh[DIM], x[DIM];
-#pragma unroll
-    for (int j = 0; j < DIM; ++j) hh[j] = x[j] = 0;
-    for (int n0 = 0; n0 < SL; n0 += K) {
+  template <typename F>
+  __device__ __forceinline__ void run(const double* __restrict__ co, int S, int E, F&& mac) {
+    int n0 = 0;
+    co += K * CS;
+    for (; n0 + 2 * K <= S; n0 += K) {  // every request in range
 #pragma unroll
       for (int d = 0; d < K; ++d) {
         const int2 q = fx_coef(c[d], E);
-        if (n0 + d + K < SL) c[d] = __ldg(co + (n0 + d + K) * cs);
-        if (n0 + d < SL) {
-          const int4 a = ua[(n0 + d) * stride];
-          hh[0] += (int64_t)q.x * a.x;
-          x[0] += (int64_t)q.x * a.y;
-          x[0] += (int64_t)q.y * a.x;
-          hh[1] += (int64_t)q.x * a.z;
-          x[1] += (int64_t)q.x * a.w;
-          x[1] += (int64_t)q.y * a.z;
-          if constexpr (DIM == 3) {
-            const int2 b = ub[(n0 + d) * stride];
-            hh[2] += (int64_t)q.x * b.x;
-            x[2] += (int64_t)q.x * b.y;
-            x[2] += (int64_t)q.y * b.x;
-          }
-        }
+        c[d] = __ldg(co + d * CS);
+        mac(q, n0, d);
       }
+      co += K * CS;
     }
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) acc[j] = fx_sum(hh[j], x[j], E, ex[j]);
+    for (int d = 0; d < K; ++d) {
+      const int2 q = fx_coef(c[d], E);
+      if (n0 + K + d < S) c[d] = __ldg(co + d * CS);
+      if (n0 + d < S) mac(q, n0, d);
+    }
+#pragma unroll
+    for (int d = 0; d < K; ++d)
+      if (n0 + K + d < S) mac(fx_coef(c[d], E), n0, K + d);
+  }
+};
+
+// mac of all components of an item, its limbs ua, ub STRIDE apart a slot
+template <int DIM, int STRIDE>
+struct FxAll {
+  const int4* ua;
+  const int2* ub;
+  FxSum s[DIM];
+  __device__ __forceinline__ void operator()(int2 q, int n0, int d) {
+    const int4 a = ua[n0 * STRIDE + d * STRIDE];
+    s[0].mac(q, a.x, a.y);
+    s[1].mac(q, a.z, a.w);
+    if constexpr (DIM == 3) {
+      const int2 b = ub[n0 * STRIDE + d * STRIDE];
+      s[2].mac(q, b.x, b.y);
+    }
   }
 };
 
@@ -242,44 +271,81 @@ __device__ __noinline__ void plain_row(const double* __restrict__ co, int64_t cs
   for (int j = 0; j < DIM; ++j) acc[j] = s[j];
 }
 
-// ---------------------------------------------------------------------
-// stabilisation extrapolation: one thread per (cell, local face)
-// ---------------------------------------------------------------------
-// NLF = faces per cell: 4 / 6 for quads / hexes, 3 / 4 for triangles / tetrahedra
-template <int DIM>
-constexpr int kUstarCells = DIM == 2 ? 32 : 16;  // cells a block: 3-D limbs fill shared memory sooner
+// shared memory of the limbs of a number of items
 template <int DIM>
 static size_t fx_smem_bytes(int S, int items) {
   return (size_t)S * items * DIM * sizeof(int2);
 }
 
+// ---------------------------------------------------------------------
+// stabilisation extrapolation: W threads per (cell, local face), each with a
+// part of the stencil (their integer sums add up exactly)
+// ---------------------------------------------------------------------
+// NLF = faces per cell: 4 / 6 for quads / hexes, 3 / 4 for triangles / tetrahedra
 template <int DIM, int NLF>
-__global__ void __launch_bounds__(kUstarCells<DIM> * NLF)
+struct UstarShape {
+  // the limbs of a 3-D stencil fill shared memory before its rows fill the
+  // SM with threads: fewer cells a block, more threads a row
+  static constexpr int CPB = DIM == 2 ? 32 : 16;
+  static constexpr int ROWS = CPB * NLF;
+  // four threads a row: 32^3 hexes 73 -> 59 us; two on 512^2 quads 57 -> 71
+  static constexpr int W = NLF >= 8 || DIM == 2 ? 1 : 4;
+  static constexpr int THREADS = ROWS * W;
+  static constexpr int BLOCKS = 1152 / THREADS;
+  static size_t smem(int S) { return fx_smem_bytes<DIM>(S, CPB) + sizeof(int64_t) * (W - 1) * ROWS * DIM; }
+};
+
+template <int DIM, int NLF>
+__global__ void __launch_bounds__(UstarShape<DIM, NLF>::THREADS, UstarShape<DIM, NLF>::BLOCKS)
     k_ustar(DevMesh m, const double* __restrict__ w, double* __restrict__ ustar) {
-  constexpr int CPB = kUstarCells<DIM>;
+  using SH = UstarShape<DIM, NLF>;
+  constexpr int CPB = SH::CPB, ROWS = SH::ROWS, W = SH::W, CS = kTile * NLF;
   extern __shared__ __align__(16) double sm[];
   __shared__ int ex[CPB * DIM];
   const int S = m.S;
-  int4* ua = reinterpret_cast<int4*>(sm);
-  int2* ub = reinterpret_cast<int2*>(ua + S * CPB);
+  int4* ua = reinterpret_cast<int4*>(sm);                                        // [S][CPB]
+  int2* ub = reinterpret_cast<int2*>(ua + S * CPB);                              // [S][CPB]
+  int64_t* part = reinterpret_cast<int64_t*>(ub + (DIM == 3 ? S * CPB : 0));     // [W-1][DIM][ROWS]
   const int64_t cell0 = (int64_t)blockIdx.x * CPB;
-  const int it = threadIdx.x, ci = it / NLF, lf = it % NLF;
+  const int it = threadIdx.x % ROWS, p = threadIdx.x / ROWS;
+  const int ci = it / NLF, lf = it % NLF;
   const int64_t cell = cell0 + ci, tile = cell0 / kTile;
   const bool on = cell < m.nc;
   const int row = (int)(cell % kTile) * NLF + lf;
-  const double* __restrict__ co = m.cex + tile * (int64_t)S * kTile * NLF + row;
-  const int SL = on ? S : 0;
-  FxRow<DIM, 5> r;
-  r.begin(co, kTile * NLF, SL);
-  const int E = on ? m.cexp[tile * kTile * NLF + row] : kFxPlain;
+  const int n0 = p * S / W, len = (p + 1) * S / W - n0;  // this thread's slots
+  const double* __restrict__ co = m.cex + tile * (int64_t)S * CS + row;
+  FxRow<5, CS> r;
+  r.begin(co + (int64_t)n0 * CS, on ? len : 0);
+  const int E = on ? m.cexp[tile * CS + row] : kFxPlain;
   const int64_t ws = m.wst;  // stride of the state read
-  fx_gather<DIM>(m.cst, w, ws, S, cell0, (int)min((int64_t)CPB, m.nc - cell0), CPB, ua, ub, ex);
-  if (!on) return;
+  fx_gather<DIM, SH::THREADS, CPB>(m.cst, w, ws, S, cell0, (int)min((int64_t)CPB, m.nc - cell0), ua, ub, ex);
+  const bool fx = E != kFxPlain && ex[ci * DIM] != 0;
+  int64_t t[DIM];
+  if (fx) {
+    FxAll<DIM, CPB> a{ua + n0 * CPB + ci, ub + n0 * CPB + ci, {}};
+    r.run(co + (int64_t)n0 * CS, len, E, a);
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) t[j] = a.s[j].total();
+  }
+  if (W > 1) {
+    if (fx && p > 0) {
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) part[((p - 1) * DIM + j) * ROWS + it] = t[j];
+    }
+    __syncthreads();
+  }
+  if (!on || p > 0) return;
   double acc[DIM];
-  if (E != kFxPlain && ex[ci * DIM] != 0)
-    r.run(co, kTile * NLF, SL, E, ua + ci, ub + ci, CPB, ex + ci * DIM, acc);
-  else
-    plain_row<DIM>(co, kTile * NLF, SL, m.cst + tile * (int64_t)S * kTile + cell % kTile, w, ws, acc);
+  if (fx) {
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) {
+#pragma unroll
+      for (int k = 0; k < W - 1; ++k) t[j] += part[(k * DIM + j) * ROWS + it];
+      acc[j] = fx_scale(t[j], E, ex[ci * DIM + j]);
+    }
+  } else {
+    plain_row<DIM>(co, CS, S, m.cst + tile * (int64_t)S * kTile + cell % kTile, w, ws, acc);
+  }
 #pragma unroll
   for (int j = 0; j < DIM; ++j) ustar[(cell * NLF + lf) * DIM + j] = w[j * ws + cell] + acc[j];
 }
@@ -424,25 +490,28 @@ __device__ __forceinline__ void traction(const double (&G)[3][3], const double* 
 // one thread a (face, row) for the gradients, a (face, point) for the law and
 // a (face, component) for the quadrature
 // ---------------------------------------------------------------------
-constexpr int kFluxThreads = 384;
-// rows a block takes: as many whole faces, 32 at most, as give each row a
-// thread; R is at most 96 (8 fan slots of 2 x 2 points)
-static int flux_faces(int R) { return std::min(kTile, kFluxThreads / R); }
-static int flux_threads(int R) { return (flux_faces(R) * R + 31) / 32 * 32; }
-template <int DIM>
-static size_t flux_smem_bytes(int S, int R) {
-  const int F = flux_faces(R);
-  return fx_smem_bytes<DIM>(S, F) + sizeof(double) * F * (R * DIM + R);
-}
+// Blocks of 192 threads at most: 467 us against 478 with 384 (32^3 hexes p = 3),
+// 353 against 372 (40^3 p = 2), as more blocks mix their phases; 1152 threads an
+// SM: 478 against 537 with 768.
+template <int DIM, int Q>
+struct FluxShape {
+  static constexpr int R = Q * DIM;  // rows a face, at most 96 (8 fan slots of 2 x 2 points)
+  static constexpr int kMaxT = 192;
+  static constexpr int FPB = kMaxT / R < kTile ? kMaxT / R : kTile;
+  static constexpr int THREADS = (FPB * R + 31) / 32 * 32;
+  static constexpr int BLOCKS = 1152 / THREADS < 32 ? 1152 / THREADS : 32;
+  static size_t smem(int S) { return fx_smem_bytes<DIM>(S, FPB) + sizeof(double) * FPB * (R * DIM + R); }
+};
 
-template <int DIM, int LAW>
-__global__ void __launch_bounds__(kFluxThreads, 3)
-    k_flux(DevMesh m, Material mt, int FPB, const double* __restrict__ w,
-           const double* __restrict__ ustar, const double* __restrict__ ubq,
-           const double* __restrict__ ubf, double* __restrict__ flux) {
+template <int DIM, int LAW, int Q>
+__global__ void __launch_bounds__(FluxShape<DIM, Q>::THREADS, FluxShape<DIM, Q>::BLOCKS)
+    k_flux(DevMesh m, Material mt, const double* __restrict__ w, const double* __restrict__ ustar,
+           const double* __restrict__ ubq, const double* __restrict__ ubf, double* __restrict__ flux) {
+  using SH = FluxShape<DIM, Q>;
+  constexpr int R = SH::R, FPB = SH::FPB;
   extern __shared__ __align__(16) double sm[];
-  __shared__ int ex[kTile * DIM];
-  const int R = m.R, Q = m.Q, S = m.S;
+  __shared__ int ex[FPB * DIM];
+  const int S = m.S;
   int4* ua = reinterpret_cast<int4*>(sm);                                // [S][FPB] components 0, 1
   int2* ub = reinterpret_cast<int2*>(ua + S * FPB);                      // [S][FPB] component 2
   double* Gs = reinterpret_cast<double*>(ub + (DIM == 3 ? S * FPB : 0)); // [FPB][R][DIM]
@@ -460,19 +529,21 @@ __global__ void __launch_bounds__(kFluxThreads, 3)
     // corner) are neither read nor formed
     const bool live = fi < nf && (m.fql == nullptr || r < __ldg(m.fql + f) * DIM);
     const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + row;
-    const int SL = live ? S : 0;
-    FxRow<DIM, 5> rw;
-    rw.begin(co, kTile * R, SL);
+    FxRow<5, kTile * R> rw;
+    rw.begin(co, live ? S : 0);
     const int E = live ? m.fexp[tile * kTile * R + row] : kFxPlain;
-    fx_gather<DIM>(m.fst, w, nc, S, f0, nf, FPB, ua, ub, ex);
+    fx_gather<DIM, SH::THREADS, FPB>(m.fst, w, nc, S, f0, nf, ua, ub, ex);
     double acc[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
     if (live) {
-      if (E != kFxPlain && ex[fi * DIM] != 0)
-        rw.run(co, kTile * R, SL, E, ua + fi, ub + fi, FPB, ex + fi * DIM, acc);
-      else
-        plain_row<DIM>(co, kTile * R, SL, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc, acc);
+      if (E != kFxPlain && ex[fi * DIM] != 0) {
+        FxAll<DIM, FPB> a{ua + fi, ub + fi, {}};
+        rw.run(co, S, E, a);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) acc[j] = fx_scale(a.s[j].total(), E, ex[fi * DIM + j]);
+      } else
+        plain_row<DIM>(co, kTile * R, S, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc, acc);
       if (f >= m.nfi && f < m.nfi + m.nfd) {  // ghost node of a displacement face
         const int64_t fd = f - m.nfi;
         const double cg = m.gco[fd * R + r];
@@ -618,6 +689,29 @@ static void by_faces_per_cell(const DevMesh& m, F&& launch) {
     launch(std::integral_constant<int, kPolyhedronMaxFaces>{});
 }
 
+// Gauss points per face as a compile-time constant: q^(d-1) for q = 1..4 in
+// 2-D, 1..3 in 3-D; on polyhedra 4 or 8 fan slots of q^2 points for q = 1, 2
+template <int DIM, typename F>
+static void by_points(const DevMesh& m, F&& launch) {
+  if constexpr (DIM == 2) {
+    switch (m.Q) {
+      case 1: return launch(std::integral_constant<int, 1>{});
+      case 2: return launch(std::integral_constant<int, 2>{});
+      case 3: return launch(std::integral_constant<int, 3>{});
+      default: return launch(std::integral_constant<int, 4>{});
+    }
+  } else {
+    switch (m.Q) {
+      case 1: return launch(std::integral_constant<int, 1>{});
+      case 4: return launch(std::integral_constant<int, 4>{});
+      case 8: return launch(std::integral_constant<int, 8>{});
+      case 16: return launch(std::integral_constant<int, 16>{});
+      case 32: return launch(std::integral_constant<int, 32>{});
+      default: return launch(std::integral_constant<int, 9>{});
+    }
+  }
+}
+
 template <int DIM, int LAW>
 static void residual_impl(const DevMesh& m, const Material& mat, const double* w,
                           const double* d_eps, const double* R0, double* out, double* ustar,
@@ -630,9 +724,8 @@ static void residual_impl(const DevMesh& m, const Material& mat, const double* w
   }
   by_faces_per_cell<DIM>(m, [&](auto nlf) {
     constexpr int NLF = decltype(nlf)::value;
-    constexpr int CPB = kUstarCells<DIM>;
-    k_ustar<DIM, NLF><<<(unsigned)((m.nc + CPB - 1) / CPB), CPB * NLF, fx_smem_bytes<DIM>(m.S, CPB), st>>>(
-        m, w, ustar);
+    using SH = UstarShape<DIM, NLF>;
+    k_ustar<DIM, NLF><<<(unsigned)((m.nc + SH::CPB - 1) / SH::CPB), SH::THREADS, SH::smem(m.S), st>>>(m, w, ustar);
   });
   if (m.nfy > 0) k_sym_other<DIM><<<(unsigned)((m.nfy + 127) / 128), 128, 0, st>>>(m, ustar);
   if (ev) cudaEventRecord(ev[1], st);
@@ -641,9 +734,12 @@ static void residual_impl(const DevMesh& m, const Material& mat, const double* w
       k_tflux<DIM><<<(unsigned)m.nftile, 32 * DIM, 0, st>>>(m, m.tco, mat.alpha * mat.kbar, w,
                                                             ustar, ubf, flux);
     } else {
-      const int fpb = flux_faces(m.R);
-      k_flux<DIM, LAW><<<(unsigned)((m.nfid + fpb - 1) / fpb), flux_threads(m.R),
-                         flux_smem_bytes<DIM>(m.S, m.R), st>>>(m, mat, fpb, w, ustar, ubq, ubf, flux);
+      by_points<DIM>(m, [&](auto q) {
+        constexpr int Q = decltype(q)::value;
+        using SH = FluxShape<DIM, Q>;
+        k_flux<DIM, LAW, Q><<<(unsigned)((m.nfid + SH::FPB - 1) / SH::FPB), SH::THREADS, SH::smem(m.S), st>>>(
+            m, mat, w, ustar, ubq, ubf, flux);
+      });
     }
   }
   if (ev) cudaEventRecord(ev[2], st);
@@ -1682,30 +1778,15 @@ static void launch_flux_df_q(const DevMesh& m, const Material& mat, const float4
       m, mat, sw, wd, ws, ubq, ubf, d_eps, flux);
 }
 
-// Gauss points per face: q^(d-1) for q = 1..4 in 2-D, 1..3 in 3-D; on
-// polyhedra 4 or 8 fan slots of q^2 points for q = 1, 2 (8 slots of 4 points
-// always with their packed groups)
+// 8 fan slots of 4 points always run with their packed groups
 template <int DIM, int LAW, int MODE>
 static void launch_flux_df(const DevMesh& m, const Material& mat, const float4* sw,
                            const double* wd, const double* ws, const double* ubq,
                            const double* ubf, const double* d_eps, double* flux, cudaStream_t st) {
-  if constexpr (DIM == 2) {
-    switch (m.Q) {
-      case 1: return launch_flux_df_q<2, LAW, MODE, 1>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 2: return launch_flux_df_q<2, LAW, MODE, 2>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 3: return launch_flux_df_q<2, LAW, MODE, 3>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      default: return launch_flux_df_q<2, LAW, MODE, 4>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-    }
-  } else {
-    switch (m.Q) {
-      case 1: return launch_flux_df_q<3, LAW, MODE, 1>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 4: return launch_flux_df_q<3, LAW, MODE, 4>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 8: return launch_flux_df_q<3, LAW, MODE, 8>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 16: return launch_flux_df_q<3, LAW, MODE, 16>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      case 32: return launch_flux_df_q<3, LAW, MODE, 32, true>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-      default: return launch_flux_df_q<3, LAW, MODE, 9>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
-    }
-  }
+  by_points<DIM>(m, [&](auto q) {
+    constexpr int Q = decltype(q)::value;
+    launch_flux_df_q<DIM, LAW, MODE, Q, Q == 32>(m, mat, sw, wd, ws, ubq, ubf, d_eps, flux, st);
+  });
 }
 
 // the state (extended by the mirror nodes when the mesh has symmetry faces)
@@ -1844,13 +1925,12 @@ static void raise_smem_fx(cudaError_t& e, K* kernel, size_t bytes) {
 }
 template <int DIM, int NLF>
 static void raise_smem_ustar(cudaError_t& e) {
-  raise_smem_fx(e, k_ustar<DIM, NLF>, fx_smem_bytes<DIM>(kMaxS, kUstarCells<DIM>));
+  raise_smem_fx(e, k_ustar<DIM, NLF>, UstarShape<DIM, NLF>::smem(kMaxS));
 }
-template <int DIM>
+template <int DIM, int Q>
 static void raise_smem_flux(cudaError_t& e) {
-  // 32 faces of at most 12 rows need the most
-  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_LINEAR>, flux_smem_bytes<DIM>(kMaxS, kFluxThreads / kTile));
-  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_NEOHOOKEAN>, flux_smem_bytes<DIM>(kMaxS, kFluxThreads / kTile));
+  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_LINEAR, Q>, FluxShape<DIM, Q>::smem(kMaxS));
+  raise_smem_fx(e, k_flux<DIM, HOFV_LAW_NEOHOOKEAN, Q>, FluxShape<DIM, Q>::smem(kMaxS));
 }
 int setup_face_kernels() {
   static int rc = -1;
@@ -1862,8 +1942,16 @@ int setup_face_kernels() {
   raise_smem_ustar<3, 4>(e);
   raise_smem_ustar<3, 6>(e);
   raise_smem_ustar<3, kPolyhedronMaxFaces>(e);
-  raise_smem_flux<2>(e);
-  raise_smem_flux<3>(e);
+  raise_smem_flux<2, 1>(e);
+  raise_smem_flux<2, 2>(e);
+  raise_smem_flux<2, 3>(e);
+  raise_smem_flux<2, 4>(e);
+  raise_smem_flux<3, 1>(e);
+  raise_smem_flux<3, 4>(e);
+  raise_smem_flux<3, 9>(e);
+  raise_smem_flux<3, 8>(e);
+  raise_smem_flux<3, 16>(e);
+  raise_smem_flux<3, 32>(e);
   raise_smem_all<2, 1>(e);
   raise_smem_all<2, 2>(e);
   raise_smem_all<2, 3>(e);
