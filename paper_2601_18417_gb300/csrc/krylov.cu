@@ -335,6 +335,10 @@ __global__ void k_cg_finish(int64_t nc, const T* __restrict__ invd, const T* __r
 //  * A cell's r, w and s are one vector load each for its neighbours; with a
 //    cell a thread (RES: at most 1024 cells a block and SM) its own values,
 //    its row of the matrix and x, p stay in registers.
+//  * In RES a neighbour of the same block is read as its new r from shared
+//    memory, after one more block barrier; only the others' r, w and s go
+//    through L2, and only cells that another block reads are stored there
+//    (45^3 hexes, 30 iterations: 293 -> 272 us).
 //  * alpha needs no quotient of the previous alpha: beta gamma / alpha_prev =
 //    beta^2 (delta - ...)_prev, gamma / beta = gamma_prev.
 // The sums keep their order (a warp's cells by shuffles in T, warps of 1024
@@ -452,8 +456,14 @@ __global__ void __launch_bounds__(kPersistThreads)
   T pg[DIM], pd[DIM];  // per-thread partials in the vector precision
   // threads j < DIM: 1 / gamma, denominator and alpha of the last iteration
   double inv_gp = 0.0, den_p = 0.0, alpha_p = 0.0;
-  // the thread's cell (RES)
-  T rD = 0, riD = 0, ro_r[DIM], wo_r[DIM], so_r[DIM], xr[DIM], pr[DIM];
+  // the thread's cell (RES): its row of the matrix and its vectors; a
+  // neighbour of the same block is an index into rs, another's is global
+  constexpr bool ROW = RES && NLF <= 6;    // the row fits in registers
+  __shared__ T rs[RES ? DIM * kPersistThreads : 1];  // the block's new r
+  T rD = 0, riD = 0, ro_r[DIM], wo_r[DIM], so_r[DIM], xr[DIM], pr[DIM], row_o[ROW ? NLF : 1];
+  int32_t row_c[ROW ? NLF : 1];
+  const int32_t cb = (int32_t)(blockIdx.x * (int64_t)blockDim.x);  // the block's first cell (RES)
+  bool seen = !RES;                        // another block reads this cell
   // ---- iteration 0: r0 = b, w0 = B D^-1 r0, x = p = 0, s_{-1} = 0
 #pragma unroll
   for (int j = 0; j < DIM; ++j) {
@@ -474,15 +484,20 @@ __global__ void __launch_bounds__(kPersistThreads)
 #pragma unroll
     for (int lf = 0; lf < NLF; ++lf) {
       const int32_t n2 = col[c * NLF + lf];
+      if (ROW) row_c[lf] = n2;
       if (n2 < 0) continue;
       const T o = mul_rn(off[c * NLF + lf], invd[n2]);
+      if (ROW) row_o[lf] = o;
+      if (RES) seen |= (uint32_t)(n2 - cb) >= (uint32_t)kPersistThreads;
 #pragma unroll
       for (int j = 0; j < DIM; ++j) ww[j] = fma(-o, (T)(-v[j * nc + n2] * inv_kbar), ww[j]);
     }
-    const T zero[DIM] = {};
-    CV::st(r[0], c, bb);
-    CV::st(w[0], c, ww);
-    CV::st(s[1], c, zero);
+    if (seen) {
+      const T zero[DIM] = {};
+      CV::st(r[0], c, bb);
+      CV::st(w[0], c, ww);
+      CV::st(s[1], c, zero);
+    }
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
       pd[j] = fma(ww[j], u[j], pd[j]);
@@ -584,54 +599,94 @@ __global__ void __launch_bounds__(kPersistThreads)
     T* sn_ = s[(i - 1) & 1];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) pg[j] = pd[j] = (T)0;
-    for (int64_t c = c0; c < nc; c += cstep) {
-      const T D = RES ? rD : -diag[c], iD = RES ? riD : invd[c];
-      T ro[DIM], wo[DIM], so[DIM], rn[DIM], s1[DIM], un[DIM], ww[DIM];
-      if (RES) {
+    if constexpr (RES) {
+      T ww[DIM], un[DIM];
+      if (c0 < nc) {
+        T rn[DIM], s1[DIM];
 #pragma unroll
-        for (int j = 0; j < DIM; ++j) ro[j] = ro_r[j], wo[j] = wo_r[j], so[j] = so_r[j];
-      } else {
+        for (int j = 0; j < DIM; ++j) {
+          s1[j] = fma(beta[j], so_r[j], wo_r[j]);
+          rn[j] = fma(-alpha[j], s1[j], ro_r[j]);
+          pr[j] = fma(ro_r[j], riD, mul_rn(beta[j], pr[j]));
+          xr[j] = fma(alpha[j], pr[j], xr[j]);
+          un[j] = mul_rn(rn[j], riD);
+          ww[j] = mul_rn(rD, un[j]);
+          pg[j] = fma(rn[j], un[j], pg[j]);
+          rs[j * kPersistThreads + threadIdx.x] = rn[j];
+          ro_r[j] = rn[j];
+          so_r[j] = s1[j];
+        }
+        if (seen) {
+          CV::st(sn_, c0, s1);
+          CV::st(rn_, c0, rn);
+        }
+      }
+      __syncthreads();
+      if (c0 < nc) {
+#pragma unroll
+        for (int lf = 0; lf < NLF; ++lf) {
+          const int32_t n2 = ROW ? row_c[ROW ? lf : 0] : col[c0 * NLF + lf];
+          if (n2 < 0) continue;
+          const T o = ROW ? row_o[ROW ? lf : 0] : mul_rn(off[c0 * NLF + lf], invd[n2]);
+          T rb[DIM];
+          const uint32_t k = (uint32_t)(n2 - cb);
+          if (k < (uint32_t)kPersistThreads) {
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) rb[j] = rs[j * kPersistThreads + k];
+          } else {
+            T wb[DIM], sb[DIM];
+            CV::ld(ro_, n2, rb);
+            CV::ld(wo_, n2, wb);
+            CV::ld(so_, n2, sb);
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) rb[j] = fma(-alpha[j], fma(beta[j], sb[j], wb[j]), rb[j]);
+          }
+#pragma unroll
+          for (int j = 0; j < DIM; ++j) ww[j] = fma(-o, rb[j], ww[j]);
+        }
+        if (seen) CV::st(wn_, c0, ww);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) {
+          pd[j] = fma(ww[j], un[j], pd[j]);
+          wo_r[j] = ww[j];
+        }
+      }
+    } else {
+      for (int64_t c = c0; c < nc; c += cstep) {
+        const T D = -diag[c], iD = invd[c];
+        T ro[DIM], wo[DIM], so[DIM], rn[DIM], s1[DIM], un[DIM], ww[DIM];
         CV::ld(ro_, c, ro);
         CV::ld(wo_, c, wo);
         CV::ld(so_, c, so);
-      }
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        s1[j] = fma(beta[j], so[j], wo[j]);
-        rn[j] = fma(-alpha[j], s1[j], ro[j]);
-        const T pold = RES ? pr[j] : pa[j * nc + c];
-        const T pv = fma(ro[j], iD, mul_rn(beta[j], pold));
-        if (RES) {
-          pr[j] = pv;
-          xr[j] = fma(alpha[j], pv, xr[j]);
-        } else {
+        for (int j = 0; j < DIM; ++j) {
+          s1[j] = fma(beta[j], so[j], wo[j]);
+          rn[j] = fma(-alpha[j], s1[j], ro[j]);
+          const T pv = fma(ro[j], iD, mul_rn(beta[j], pa[j * nc + c]));
           pa[j * nc + c] = pv;
           xa[j * nc + c] = fma(alpha[j], pv, xa[j * nc + c]);
+          un[j] = mul_rn(rn[j], iD);
+          ww[j] = mul_rn(D, un[j]);
+          pg[j] = fma(rn[j], un[j], pg[j]);
         }
-        un[j] = mul_rn(rn[j], iD);
-        ww[j] = mul_rn(D, un[j]);
-        pg[j] = fma(rn[j], un[j], pg[j]);
-      }
-      CV::st(sn_, c, s1);
-      CV::st(rn_, c, rn);
+        CV::st(sn_, c, s1);
+        CV::st(rn_, c, rn);
 #pragma unroll
-      for (int lf = 0; lf < NLF; ++lf) {
-        const int32_t n2 = col[c * NLF + lf];
-        if (n2 < 0) continue;
-        const T o = mul_rn(off[c * NLF + lf], invd[n2]);
-        T rb[DIM], wb[DIM], sb[DIM];
-        CV::ld(ro_, n2, rb);
-        CV::ld(wo_, n2, wb);
-        CV::ld(so_, n2, sb);
+        for (int lf = 0; lf < NLF; ++lf) {
+          const int32_t n2 = col[c * NLF + lf];
+          if (n2 < 0) continue;
+          const T o = mul_rn(off[c * NLF + lf], invd[n2]);
+          T rb[DIM], wb[DIM], sb[DIM];
+          CV::ld(ro_, n2, rb);
+          CV::ld(wo_, n2, wb);
+          CV::ld(so_, n2, sb);
 #pragma unroll
-        for (int j = 0; j < DIM; ++j)
-          ww[j] = fma(-o, fma(-alpha[j], fma(beta[j], sb[j], wb[j]), rb[j]), ww[j]);
-      }
-      CV::st(wn_, c, ww);
+          for (int j = 0; j < DIM; ++j)
+            ww[j] = fma(-o, fma(-alpha[j], fma(beta[j], sb[j], wb[j]), rb[j]), ww[j]);
+        }
+        CV::st(wn_, c, ww);
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        pd[j] = fma(ww[j], un[j], pd[j]);
-        if (RES) ro_r[j] = rn[j], wo_r[j] = ww[j], so_r[j] = s1[j];
+        for (int j = 0; j < DIM; ++j) pd[j] = fma(ww[j], un[j], pd[j]);
       }
     }
   }
