@@ -367,6 +367,7 @@ void hofv_destroy(hofv_ctx* c) {
   else cudaDeviceSynchronize();
   free_built(c);
   if (c->cap) cudaStreamDestroy(c->cap);
+  if (c->h_kry) cudaFreeHost(c->h_kry);
   delete c;
 }
 
@@ -1252,6 +1253,20 @@ struct ArnoldiKey {
            V == o.V && Z == o.Z && w == o.w && dh == o.dh && ld == o.ld && dstride == o.dstride;
   }
 };
+// The projections and the norm of a step (up to 2 * 102 + 1 doubles) and the
+// two error flags come back in one page of pinned memory with one wait.  As four
+// copies to pageable memory, each waiting by itself, they left the device idle
+// for a quarter of a solve on 12^3 hexes (7.67 -> 5.73 ms with this).
+constexpr int kKryHost = 256;                // doubles; the flags lie in the last one
+static int check_flags(hofv_ctx* c, const int* flags);
+static int read_step(hofv_ctx* c, const double* dh, int count) {
+  int* flags = reinterpret_cast<int*>(c->h_kry + kKryHost - 1);
+  HOFV_CUDA(c, cudaMemcpyAsync(c->h_kry, dh, sizeof(double) * count, cudaMemcpyDeviceToHost, c->stream));
+  HOFV_CUDA(c, cudaMemcpyAsync(flags, c->d_bar + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
+  return check_flags(c, flags);
+}
+
 struct GraphCache {
   std::vector<std::pair<ArnoldiKey, cudaGraphExec_t>> items;
   bool broken = false;  // a capture failed once: launch directly from then on
@@ -1345,10 +1360,11 @@ static int arnoldi_device(hofv_ctx* c, const hofv_solve_opts& o, const ArnoldiKe
 // host-side FGMRES state for one linear solve J x = b
 struct Fgmres {
   std::vector<double> H;   // [(m+1) x m] column-major
-  std::vector<double> cs, sn, g, y, hbuf;
+  std::vector<double> cs, sn, g, y;
 };
 
 static int ensure_krylov(hofv_ctx* c, int m) {
+  if (!c->h_kry) HOFV_CUDA(c, cudaMallocHost(&c->h_kry, sizeof(double) * kKryHost));
   if (c->kry_m >= m) return 0;
   const int64_t n = c->nc * c->dim;
   dev_free(c, c->d_V);
@@ -1409,7 +1425,6 @@ static int fgmres(hofv_ctx* c, const hofv_solve_opts& o, const double* u, const 
   F.sn.assign(m, 0.0);
   F.g.assign(m + 1, 0.0);
   F.y.assign(m, 0.0);
-  F.hbuf.assign(2 * (m + 2), 0.0);
   HOFV_CUDA(c, cudaMemsetAsync(x, 0, sizeof(double) * n, c->stream));
   HOFV_CUDA(c, cudaMemcpyAsync(r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
   TRY(ensure_jv_cache(c, u, Ru));
@@ -1447,18 +1462,17 @@ static int fgmres(hofv_ctx* c, const hofv_solve_opts& o, const double* u, const 
         launch_dots(V, n, w, j + 1, n, c->d_red, c->d_count, dh + (m + 2), c->red_blocks, c->stream, 0);
         launch_multi_axpy(w, V, dh + (m + 2), j + 1, n, n, c->stream);
         launch_norm2(w, n, c->d_red, c->d_count, dh + 2 * (m + 2), c->red_blocks, c->stream);
+        launch_scale_copy(V + (int64_t)(j + 1) * n, w, dh + 2 * (m + 2), 1, n, c->stream);
       } else {
-        const ArnoldiKey key{c->gen, oc.precond, oc.inner_iters, j, 0, 0, u, Ru, V, Z, w, dh,
+        // v_{j+1} = w / |w| follows at once (with |w| = 0 it is never read)
+        const ArnoldiKey key{c->gen, oc.precond, oc.inner_iters, j, 0, 1, u, Ru, V, Z, w, dh,
                              n, m + 2};
         TRY(arnoldi_device(c, oc, key, st));
       }
       st->residual_evals++;
-      HOFV_CUDA(c, cudaMemcpyAsync(F.hbuf.data(), dh, sizeof(double) * 2 * (m + 2),
-                                   cudaMemcpyDeviceToHost, c->stream));
-      double hn = 0.0;
-      HOFV_CUDA(c, cudaMemcpyAsync(&hn, dh + 2 * (m + 2), sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-      HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
-      TRY(check_pc_barrier(c));
+      TRY(read_step(c, dh, 2 * (m + 2) + 1));
+      const double* hbuf = c->h_kry;
+      const double hn = hbuf[2 * (m + 2)];
       if (!std::isfinite(hn) && cycle_gnn) {
         // learned preconditioner failed: drop this cycle, continue with AJ
         oc.precond = HOFV_PC_AJ32;
@@ -1468,9 +1482,8 @@ static int fgmres(hofv_ctx* c, const hofv_solve_opts& o, const double* u, const 
       }
       if (!std::isfinite(hn)) return fail(c, HOFV_ENAN, "non-finite value in the Krylov basis");
       double* Hc = F.H.data() + (size_t)j * (m + 1);
-      for (int i = 0; i <= j; ++i) Hc[i] = F.hbuf[i] + F.hbuf[(m + 2) + i];
+      for (int i = 0; i <= j; ++i) Hc[i] = hbuf[i] + hbuf[(m + 2) + i];
       Hc[j + 1] = hn;
-      if (hn > 0.0) launch_scale_copy(V + (int64_t)(j + 1) * n, w, dh + 2 * (m + 2), 1, n, c->stream);
       for (int i = 0; i < j; ++i) {  // previous rotations
         const double t = F.cs[i] * Hc[i] + F.sn[i] * Hc[i + 1];
         Hc[i + 1] = -F.sn[i] * Hc[i] + F.cs[i] * Hc[i + 1];
@@ -1781,11 +1794,8 @@ extern "C" int hofv_arnoldi_step(hofv_ctx* c, const double* u, const double* Ru,
   const ArnoldiKey key{c->gen, kind, inner_iters, j, 1, 1, u, Ru, V, Z, w, dh, ld, k};
   TRY(ensure_jv_cache(c, u, Ru));
   TRY(arnoldi_device(c, o, key, &st));
-  std::vector<double> hb((size_t)(2 * k + 1));
-  HOFV_CUDA(c, cudaMemcpyAsync(hb.data(), dh, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost,
-                               c->stream));
-  HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
-  TRY(check_pc_barrier(c));
+  TRY(read_step(c, dh, 2 * k + 1));
+  const double* hb = c->h_kry;
   for (int i = 0; i < k; ++i) h[i] = hb[i] + hb[k + i];
   h[k] = hb[2 * k];
   if (!std::isfinite(h[k])) return fail(c, HOFV_ENAN, "non-finite value in the Arnoldi step");
@@ -1827,16 +1837,13 @@ extern "C" int hofv_force_scale(hofv_ctx* c, const double* u, double* fs) {
 }
 
 namespace hofv {
-int check_pc_barrier(hofv_ctx* c) {
-  if (!c->d_bar) return 0;
-  int err = 0;
-  HOFV_CUDA(c, cudaMemcpy(&err, c->d_bar + 2, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
+// the flags as read from d_bar + 2: the grid barrier's, the face kernels'
+static int check_flags(hofv_ctx* c, const int* flags) {
+  if (flags[0]) {
     HOFV_CUDA(c, cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)));
     return fail(c, HOFV_ECUDA, "approximate-Jacobian solve: grid barrier timed out");
   }
-  HOFV_CUDA(c, cudaMemcpy(&err, c->d_bar + 3, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
+  if (flags[1]) {
     HOFV_CUDA(c, cudaMemset(c->d_bar + 3, 0, sizeof(unsigned int)));
     return fail(c, HOFV_ECUDA, "face kernel: a shared-memory copy did not complete in time");
   }

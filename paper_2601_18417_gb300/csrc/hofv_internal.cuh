@@ -223,6 +223,7 @@ struct hofv_ctx {
   double* d_Z = nullptr;            // [m][n]
   double* d_kvec = nullptr;         // work vectors
   double* d_h = nullptr;            // [m+2] projections
+  double* h_kry = nullptr;          // pinned: a step's projections and flags (api.cu)
   // ---- learned preconditioner ----
   void* gnn = nullptr;
   // ---- multigrid hierarchy of the approximate Jacobian ----
@@ -371,9 +372,6 @@ void launch_combine(double* x, const double* Z, const double* y, int k, int64_t 
                     cudaStream_t st);
 void launch_axpby(double* y, double a, const double* x, double b, int64_t n, cudaStream_t st);
 int aj_precondition(hofv_ctx* c, int kind, int iters, const double* v, double* z);
-// error of a timed-out persistent-CG grid barrier since the last check
-// (reads the flag: call after a stream synchronisation), then clears it
-int check_pc_barrier(hofv_ctx* c);
 // bounded-wait self-test of the grid barrier (see hofv_selftest_barrier)
 int barrier_selftest(hofv_ctx* c, int* timed_out);
 
