@@ -349,35 +349,35 @@ unsigned grid_for(int64_t n) {
 
 // ---- V-cycle kernels (all components per thread, component stride n) ----
 
-// b as stored (float), or as the caller's FP64 right-hand side times a scale
-template <typename TB>
-__device__ __forceinline__ float ldb(const TB* b, int64_t k, double bs) {
-  if constexpr (sizeof(TB) == 8)
-    return (float)(b[k] * bs);
-  else
-    return b[k];
+// b = v * bs in FP32: once a value, as the product and the conversion hold the
+// FP64 pipe for 16 cycles each.  When the finest smoothers made them for every
+// neighbour they read, they took 27.5 and 7.1 us on 64^3 hexes, now 8.1, 5.5 and
+// 4 here
+__global__ void k_to_float(int64_t n, const double* __restrict__ v, double bs, float* __restrict__ b) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    b[i] = (float)(v[i] * bs);
 }
 
 // x = W b (W = omega D^-1), r = b - B x
-template <int DIM, typename TB = float>
+template <int DIM>
 __global__ void k_pre(int64_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                       const float* __restrict__ va, const float* __restrict__ dg,
-                      const float* __restrict__ dinv, const TB* __restrict__ b, double bs,
-                      float* x, float* r) {
+                      const float* __restrict__ dinv, const float* __restrict__ b, float* x,
+                      float* r) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float wi = dinv[i], di = dg[i];
     float bi[DIM], s[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
-      bi[j] = ldb(b, j * n + i, bs);
+      bi[j] = b[j * n + i];
       s[j] = di * wi * bi[j];
     }
     for (int32_t k = rp[i]; k < rp[i + 1]; ++k) {
       const int32_t c = ci[k];
       const float a = va[k] * dinv[c];
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) s[j] += a * ldb(b, j * n + c, bs);
+      for (int j = 0; j < DIM; ++j) s[j] += a * b[j * n + c];
     }
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
@@ -409,10 +409,10 @@ __global__ void k_csr_apply(int64_t nrow, int64_t nin, const int32_t* __restrict
 }
 
 // y = x + W (b - B x)
-template <int DIM, typename TB = float, typename TY = float>
+template <int DIM, typename TY = float>
 __global__ void k_post(int64_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                        const float* __restrict__ va, const float* __restrict__ dg,
-                       const float* __restrict__ dinv, const TB* __restrict__ b, double bs,
+                       const float* __restrict__ dinv, const float* __restrict__ b,
                        const float* __restrict__ x, TY* y) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -421,7 +421,7 @@ __global__ void k_post(int64_t n, const int32_t* __restrict__ rp, const int32_t*
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
       xi[j] = x[j * n + i];
-      s[j] = ldb(b, j * n + i, bs) - di * xi[j];
+      s[j] = b[j * n + i] - di * xi[j];
     }
     for (int32_t k = rp[i]; k < rp[i + 1]; ++k) {
       const int32_t c = ci[k];
@@ -561,8 +561,7 @@ void pre(const Level& L, const float* b, float* x, float* r, cudaStream_t st) {
   if (L.a_warp)
     k_pre_w<DIM><<<grid_warps(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, x, r);
   else
-    k_pre<DIM><<<grid_for(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, 1.0, x,
-                                                   r);
+    k_pre<DIM><<<grid_for(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, x, r);
 }
 
 template <int DIM>
@@ -571,8 +570,7 @@ void post(const Level& L, const float* b, const float* x, float* y, cudaStream_t
     k_post_w<DIM><<<grid_warps(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, x,
                                                         y);
   else
-    k_post<DIM><<<grid_for(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, 1.0, x,
-                                                    y);
+    k_post<DIM><<<grid_for(L.n), kThreads, 0, st>>>(L.n, L.rp, L.ci, L.va, L.dg, L.dinv, b, x, y);
 }
 
 template <int DIM, bool ADD>
@@ -852,18 +850,16 @@ void run(hofv_ctx* c, Mg& g, int iters, const double* v, double* zout) {
   const Level& L = g.L[0];
   const unsigned gb = (unsigned)g.blocks;
   if (iters == 1 && g.L.size() > 1) {
-    // one V-cycle applied to b = -v / Kbar, read and written in FP64 by the
-    // finest level's smoothers (the flexible outer solver absorbs the
-    // missing CG step length: it only scales z)
+    // one V-cycle applied to b = -v / Kbar, written in FP64 by the finest
+    // level's smoother (the flexible outer solver absorbs the missing CG step
+    // length: it only scales z)
     const Level& C = g.L[1];
-    const double bs = -1.0 / c->mat.kbar;
-    k_pre<DIM, double><<<grid_for(n), kThreads, 0, st>>>(n, L.rp, L.ci, L.va, L.dg, L.dinv, v, bs,
-                                                         L.x, L.r);
+    k_to_float<<<grid_for(DIM * n), kThreads, 0, st>>>(DIM * n, v, -1.0 / c->mat.kbar, L.b);
+    k_pre<DIM><<<grid_for(n), kThreads, 0, st>>>(n, L.rp, L.ci, L.va, L.dg, L.dinv, L.b, L.x, L.r);
     apply<DIM, false>(L.r_warp, C.n, n, L.rrp, L.rci, L.rva, L.r, C.b, st);
     vcycle<DIM>(g, 1, C.b, C.y, st);
     apply<DIM, true>(L.p_warp, n, C.n, L.prp, L.pci, L.pva, C.y, L.x, st);
-    k_post<DIM, double, double><<<grid_for(n), kThreads, 0, st>>>(n, L.rp, L.ci, L.va, L.dg,
-                                                                  L.dinv, v, bs, L.x, zout);
+    k_post<DIM, double><<<grid_for(n), kThreads, 0, st>>>(n, L.rp, L.ci, L.va, L.dg, L.dinv, L.b, L.x, zout);
     return;
   }
   k_cg_start<DIM><<<grid_for(DIM * n), kThreads, 0, st>>>(n, v, 1.0 / c->mat.kbar, g.r, g.x);
