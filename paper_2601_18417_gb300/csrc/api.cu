@@ -43,6 +43,7 @@ DevMesh dev_mesh(const hofv_ctx* c) {
   m.S = c->S;
   m.Q = c->Q;
   m.R = c->Q * c->dim;
+  m.sms = c->sm_count;
   m.nc = c->nc;
   m.nf = c->nf;
   m.nfi = c->nfi;

@@ -43,6 +43,7 @@ __device__ __forceinline__ double inv_cbrt(double J) {
 // kernels.  All pointers are device addresses owned by the context.
 struct DevMesh {
   int dim, nlf, S, Q, R;          // R = Q * dim rows per face
+  int sms;                        // streaming multiprocessors of the device
   int64_t nc, nf, nfi, nfd, nft;
   int64_t nfid;                   // internal + displacement faces
   int64_t nftile;                 // face tiles of kTile (internal + disp)

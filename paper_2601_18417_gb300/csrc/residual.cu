@@ -1247,8 +1247,9 @@ struct UsShape {
   static constexpr int RPG = NLF >= 8 ? 4 : NLF;   // rows a warp takes
   static constexpr int NG = NLF / RPG;             // row groups
   static constexpr bool SPARSE = NLF >= 8;         // cells with empty face slots
-  static constexpr int split(int S) { return NLF == 16 ? 2 : S > 32 ? 4 : 2; }
-  static constexpr int THREADS = NLF >= 8 ? 256 : 128;  // at most
+  // few: no tile for each SM (13^3 hexes 15.9 -> 10.5 us with eight)
+  static constexpr int split(int S, bool few) { return NLF == 16 ? 2 : S <= 32 ? 2 : few && NLF < 8 ? 8 : 4; }
+  static constexpr int THREADS = 256;              // at most
 };
 
 template <int DIM, int NLF>
@@ -1760,7 +1761,7 @@ static void launch_ustar_df(const DevMesh& m, const float4* sw, const double* w,
   by_faces_per_cell<DIM>(m, [&](auto nlf) {
     constexpr int NLF = decltype(nlf)::value;
     using SH = UsShape<NLF>;
-    const int W = SH::split(m.S);
+    const int W = SH::split(m.S, m.nctile <= m.sms);
     k_ustar_df<DIM, NLF><<<(unsigned)m.nctile, 32 * SH::NG * W, sizeof(float2) * W * NLF * DIM * 33, st>>>(
         m, sw, w, out);
   });
