@@ -1130,14 +1130,13 @@ int hofv_residual(hofv_ctx* c, const double* u, double* R) {
   return HOFV_OK;
 }
 
-// Jv with ||u|| already in d_scal[0]: computes ||v||, eps, w = u + eps v and
-// (R(w) - Ru) / eps into Jv.  eps stays in d_scal[2].
+// Jv: computes ||v||, ||u|| (with_unorm; else it lies in d_scal[0]), eps,
+// w = u + eps v and (R(w) - Ru) / eps into Jv.  eps stays in d_scal[2].
 static int jvp_impl(hofv_ctx* c, const double* u, const double* Ru, const double* v, double* Jv,
-                    cudaEvent_t* ev = nullptr) {
+                    bool with_unorm = false, cudaEvent_t* ev = nullptr) {
   const int64_t n = c->nc * c->dim;
   double* sc = c->d_scal;
-  launch_norm2(v, n, c->d_red, c->d_count, sc + 1, c->red_blocks, c->stream);
-  launch_jv_eps(sc + 0, sc + 1, sc + 2, c->stream);
+  launch_jv_norms(v, with_unorm ? u : nullptr, n, c->d_red, c->d_count, sc, c->red_blocks, c->stream);
   if (c->prec == HOFV_PREC_DF64) {  // the caller made the linearisation cache valid
     launch_jv_df(dev_mesh(c), c->mat, v, sc + 2, Jv, c->d_flux, c->stream, ev);
     HOFV_CUDA(c, cudaGetLastError());
@@ -1154,10 +1153,8 @@ int hofv_jvp(hofv_ctx* c, const double* u, const double* Ru, const double* v, do
              double* eps_used) {
   TRY(check_eval(c));
   if (!u || !Ru || !v || !Jv) return fail(c, HOFV_EINVAL, "null vector");
-  const int64_t n = c->nc * c->dim;
-  launch_norm2(u, n, c->d_red, c->d_count, c->d_scal + 0, c->red_blocks, c->stream);
   TRY(ensure_jv_cache(c, u, Ru));
-  TRY(jvp_impl(c, u, Ru, v, Jv));
+  TRY(jvp_impl(c, u, Ru, v, Jv, true));
   if (eps_used) {
     HOFV_CUDA(c, cudaMemcpyAsync(eps_used, c->d_scal + 2, sizeof(double), cudaMemcpyDeviceToHost,
                                  c->stream));
@@ -1170,12 +1167,10 @@ int hofv_jvp_timed(hofv_ctx* c, const double* u, const double* Ru, const double*
                    float* ms) {
   TRY(check_eval(c));
   if (!u || !Ru || !v || !Jv || !ms) return fail(c, HOFV_EINVAL, "null argument");
-  const int64_t n = c->nc * c->dim;
-  launch_norm2(u, n, c->d_red, c->d_count, c->d_scal + 0, c->red_blocks, c->stream);
   TRY(ensure_jv_cache(c, u, Ru));
   cudaEvent_t ev[4];
   for (int i = 0; i < 4; ++i) HOFV_CUDA(c, cudaEventCreate(&ev[i]));
-  const int rc = jvp_impl(c, u, Ru, v, Jv, ev);
+  const int rc = jvp_impl(c, u, Ru, v, Jv, true, ev);
   cudaError_t e = rc == 0 ? cudaEventSynchronize(ev[3]) : cudaSuccess;
   for (int i = 0; i < 3 && rc == 0 && e == cudaSuccess; ++i)
     e = cudaEventElapsedTime(&ms[i], ev[i], ev[i + 1]);
@@ -1295,8 +1290,7 @@ static int arnoldi_launch(hofv_ctx* c, const hofv_solve_opts& o, const ArnoldiKe
   double* Zj = Z + (int64_t)k.j * k.ld;
   const int nv = k.j + 1;
   TRY(apply_pc(c, o, Vj, Zj, st));
-  if (k.with_unorm) launch_norm2(k.u, n, c->d_red, c->d_count, c->d_scal + 0, c->red_blocks, c->stream);
-  TRY(jvp_impl(c, k.u, k.Ru, Zj, w));
+  TRY(jvp_impl(c, k.u, k.Ru, Zj, w, k.with_unorm));
   launch_dots(V, k.ld, w, nv, n, c->d_red, c->d_count, dh, c->red_blocks, c->stream, 0);
   launch_multi_axpy(w, V, dh, nv, n, k.ld, c->stream);
   launch_dots(V, k.ld, w, nv, n, c->d_red, c->d_count, dh + k.dstride, c->red_blocks, c->stream, 0);

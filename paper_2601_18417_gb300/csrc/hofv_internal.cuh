@@ -361,7 +361,9 @@ void launch_dots(const double* X, int64_t ldx, const double* y, int nvec, int64_
                  unsigned int* count, double* out, int blocks, cudaStream_t st, int mode);
 void launch_norm2(const double* x, int64_t n, double* red, unsigned int* count, double* out,
                   int blocks, cudaStream_t st);
-void launch_jv_eps(const double* u_norm, const double* v_norm, double* eps, cudaStream_t st);
+// sc[1] = |v|, sc[0] = |u| (kept where u is null), sc[2] = the step eps of Jv
+void launch_jv_norms(const double* v, const double* u, int64_t n, double* red, unsigned int* count, double* sc,
+                     int blocks, cudaStream_t st);
 // y = x + sign * alpha[0] * v
 void launch_waxpy_dev(double* y, const double* x, const double* v, const double* alpha,
                       double sign, int64_t n, cudaStream_t st);
