@@ -513,11 +513,11 @@ def step_section(args, wl, mesh, ctx, lay, u_ex, precision, rank, ws, peaks_dev,
     ko = np.array([ctx.residual_timed(u, Ru) for _ in range(10)])
     ctx.set_precision(prec)
     ctx.residual(u, Ru)
-    # per step: the preconditioner (one V-cycle: 4 launches per level above the
-    # coarsest, 1 on it) + norm (1) + Jv (norm, eps, split / axpy, 3 residual
-    # kernels) + CGS2 (2 multi-dots, 2 multi-axpys) + norm + scale
+    # per step: the preconditioner (the conversion and one V-cycle: 4 launches
+    # per level above the coarsest, 1 on it) + Jv (norms and eps, split / axpy, 3
+    # residual kernels) + CGS2 (2 multi-dots, 2 multi-axpys) + norm + scale
     assert MG_INNER == 1 and mg["levels"] > 1
-    launches = (4 * (mg["levels"] - 1) + 1) + 1 + 6 + 4 + 2
+    launches = 1 + (4 * (mg["levels"] - 1) + 1) + 5 + 4 + 2
     return {"ms": ms, "u": u, "Ru": Ru, "mg": mg, "roofline": roofline, "e2e": e2e,
             "launches": launches,
             "step_ms_no_graph": {"ms_per_step": ms_direct, "value": nc / (ms_direct * 1e-3) / 1e6},
