@@ -298,10 +298,11 @@ int hofv_set_contraction(hofv_ctx* ctx, int on);
    gradient at every face Gauss point, eq. faceQuadGrad, and the
    extrapolated face values of the stabilisation, eq. alphaJump).
    HOFV_PREC_FP64 (default) takes FP64 coefficients and values and sums their
-   products in 64-bit fixed point: each slot's error is at most 2^-54 of the
-   row's largest coefficient times the stencil's largest value (FP64 fused
-   multiply-adds, which round at 2^-53 of every partial sum, where either is
-   not finite or beyond about 1e+-145).  HOFV_PREC_DF64 stores each coefficient as a pair of floats (hi, lo), hi + lo its value
+   products in 64-bit fixed point: each slot's error is at most 2^-53 of the
+   row's largest coefficient times the stencil's largest value, where FP64
+   fused multiply-adds round at 2^-53 of every partial sum (they are used where
+   either is not finite or beyond about 1e+-145).  HOFV_PREC_DF64 stores
+   each coefficient as a pair of floats (hi, lo), hi + lo its value
    rounded to 48 significant bits, splits the state exactly into three
    floats, and forms each product exactly (TwoProduct by FMA, Dekker 1971)
    and the sums with TwoSum and a compensation term (Dot2, Ogita, Rump &

@@ -33,7 +33,7 @@ SCHEMES = [(2, 9, 1, 1), (2, 33, 2, 2), (2, 17, 3, 3), (2, 12, 3, 4), (3, 5, 1, 
 @pytest.mark.parametrize("dim,n,p,q1", SCHEMES)
 @pytest.mark.parametrize("spread", [0, 40])
 def test_against_oracle(dim, n, p, q1, spread):
-    """A slot's error is at most 2^-54 of its face's largest coefficient times
+    """A slot's error is at most 2^-53 of its face's largest coefficient times
     its largest value, below the bound of an FP64 sum: the tolerance is the
     1e-12 of the force scale that FP64 residuals are held to elsewhere."""
     pb, ctx = _problem(dim, n, p, q1)
