@@ -301,7 +301,7 @@ int run_aj_rows(hofv_ctx* c);
 
 // ---- residual kernels (residual.cu) ----
 // R = residual(w) where w = u (+ eps * v when v != nullptr, eps read from
-// *d_eps on the device); when R0 != nullptr the output is (R(w) - R0) / eps.
+// *d_eps on the device, 1 / eps beside it); when R0 != nullptr the output is (R(w) - R0) / eps.
 void launch_residual(const DevMesh& m, const Material& mat, const double* u, const double* v,
                      const double* d_eps, const double* R0, double* out, double* ustar,
                      double* flux, const double* ubq, const double* ubf, const double* src,
@@ -361,7 +361,7 @@ void launch_dots(const double* X, int64_t ldx, const double* y, int nvec, int64_
                  unsigned int* count, double* out, int blocks, cudaStream_t st, int mode);
 void launch_norm2(const double* x, int64_t n, double* red, unsigned int* count, double* out,
                   int blocks, cudaStream_t st);
-// sc[1] = |v|, sc[0] = |u| (kept where u is null), sc[2] = the step eps of Jv
+// sc[1] = |v|, sc[0] = |u| (kept where u is null), sc[2] = the step eps of Jv, sc[3] = 1 / eps
 void launch_jv_norms(const double* v, const double* u, int64_t n, double* red, unsigned int* count, double* sc,
                      int blocks, cudaStream_t st);
 // y = x + sign * alpha[0] * v

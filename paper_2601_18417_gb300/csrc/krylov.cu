@@ -16,25 +16,95 @@ namespace hofv {
 
 constexpr int kRedThreads = 256;
 
-// out[k] = x_k . y for k = blockIdx.y; x_k = X + k * ldx
-__global__ void k_mdot(const double* __restrict__ X, int64_t ldx, const double* __restrict__ y,
-                       int64_t n, double* red, unsigned int* count, double* out, int mode) {
-  __shared__ double sh[32];
-  const int k = blockIdx.y;
-  const double* x = X + k * ldx;
-  double s = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    s = fma(x[i], y[i], s);
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) red[k * gridDim.x + blockIdx.x] = s;
-  if (last_block(count + k, gridDim.x)) {
+// Sums of NV values a thread over the block, value k in lane 0 of warp k: the
+// warps' lanes first, one warp a value, so that FP64 additions, which hold
+// the pipe for 16 cycles a warp, are 13 a value and not 40.
+template <int NV>
+__device__ __forceinline__ double block_sums(const double (&v)[NV], double* sh) {
+  constexpr int NW = kRedThreads / 32;
+  static_assert(NV <= NW, "a warp a value");
+#pragma unroll
+  for (int k = 0; k < NV; ++k) sh[k * kRedThreads + threadIdx.x] = v[k];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double t = 0.0;
+  if (wid < NV) {
+    double q[NW];
+#pragma unroll
+    for (int i = 0; i < NW; ++i) q[i] = sh[wid * kRedThreads + i * 32 + lane];
+#pragma unroll
+    for (int h = NW / 2; h > 0; h /= 2)  // pairwise: the additions' latency counts
+#pragma unroll
+      for (int i = 0; i < h; ++i) q[i] += q[i + h];
+    t = q[0];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  return t;
+}
+
+// True in all threads of the last of n blocks to come here; the writers of what
+// that block reads have each put a fence behind their writes.
+__device__ __forceinline__ bool last_to_come(unsigned int* count, unsigned int n) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(count, 1u) == n - 1;
     __threadfence();
-    const double t = warp0_sum(red + k * gridDim.x, gridDim.x);
-    if (threadIdx.x == 0) {
-      out[k] = mode == 1 ? sqrt(t) : t;
-      count[k] = 0;
+  }
+  __syncthreads();
+  return last;
+}
+
+// out[k0 + k] = x_k . y for NV vectors x_k = X + (k0 + k) * ldx
+template <int NV>
+__device__ __forceinline__ void mdot(const double* __restrict__ X, int64_t ldx, const double* __restrict__ y,
+                                     int64_t n, int k0, double* red, unsigned int* count, double* out, int mode,
+                                     double* sh) {
+  double s[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) s[k] = 0.0;
+  const double* __restrict__ x = X + k0 * ldx;
+#pragma unroll 4
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const double yi = y[i];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) s[k] = fma(x[k * ldx + i], yi, s[k]);
+  }
+  const double t = block_sums<NV>(s, sh);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (wid < NV && lane == 0) {
+    __stcg(red + (k0 + wid) * gridDim.x + blockIdx.x, t);
+    __threadfence();
+  }
+  if (last_to_come(count + blockIdx.y, gridDim.x)) {
+    if (wid < NV) {  // a warp a vector, in block order
+      const double* r = red + (k0 + wid) * gridDim.x;
+      double a = 0.0;
+#pragma unroll 8
+      for (unsigned int b = lane; b < gridDim.x; b += 32) a += __ldcg(r + b);
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) out[k0 + wid] = mode == 1 ? sqrt(a) : a;
     }
+    if (threadIdx.x == 0) count[blockIdx.y] = 0;
+  }
+}
+
+// kMdot vectors a block.  The pass is bound by the FP64 pipe (22 us for 16
+// vectors of 64^3 x 3); one vector a block with a shuffle tree in each warp
+// took 35 us (27 on 512^2 x 2, pipe 15), this 31 (23): y is read a quarter as often
+// and the reductions are a tenth of the FP64 instructions.
+constexpr int kMdot = 4;
+__global__ void __launch_bounds__(kRedThreads)
+    k_mdot(const double* __restrict__ X, int64_t ldx, const double* __restrict__ y, int nvec, int64_t n,
+           double* red, unsigned int* count, double* out, int mode) {
+  __shared__ double sh[kMdot * kRedThreads];
+  const int k0 = blockIdx.y * kMdot;
+  switch (min(nvec - k0, kMdot)) {
+    case 1: return mdot<1>(X, ldx, y, n, k0, red, count, out, mode, sh);
+    case 2: return mdot<2>(X, ldx, y, n, k0, red, count, out, mode, sh);
+    case 3: return mdot<3>(X, ldx, y, n, k0, red, count, out, mode, sh);
+    default: return mdot<kMdot>(X, ldx, y, n, k0, red, count, out, mode, sh);
   }
 }
 
@@ -42,8 +112,8 @@ void launch_dots(const double* X, int64_t ldx, const double* y, int nvec, int64_
                  unsigned int* count, double* out, int blocks, cudaStream_t st, int mode) {
   // few blocks per vector: every block ends in FP64 warp reductions
   blocks = (int)std::min<int64_t>(std::max(blocks / 4, 1), (n + kRedThreads - 1) / kRedThreads);
-  dim3 grid((unsigned)blocks, (unsigned)nvec);
-  k_mdot<<<grid, kRedThreads, 0, st>>>(X, ldx, y, n, red, count, out, mode);
+  dim3 grid((unsigned)blocks, (unsigned)((nvec + kMdot - 1) / kMdot));
+  k_mdot<<<grid, kRedThreads, 0, st>>>(X, ldx, y, nvec, n, red, count, out, mode);
 }
 
 void launch_norm2(const double* x, int64_t n, double* red, unsigned int* count, double* out,
@@ -52,9 +122,11 @@ void launch_norm2(const double* x, int64_t n, double* red, unsigned int* count, 
 }
 
 // sc[1] = ||v||, sc[0] = ||u|| (slice 1, where the launch has it), then
-// sc[2] = eps = sqrt(2^-52) (1 + ||u||) / ||v|| (1 if v = 0).  One launch for
+// sc[2] = eps = sqrt(2^-52) (1 + ||u||) / ||v|| (1 if v = 0) and sc[3] = 1 / eps,
+// which the assembly would divide out in every thread.  One launch for
 // what took three, each mostly latency: a product on 13^3 hexes 92 -> 84 us.
-// The norms' sums are those of k_mdot.
+// A step's rounding passes through eps to the whole difference quotient, so the
+// sums are in the order of separate norms, block_sum's.
 __global__ void k_jv_norms(const double* __restrict__ v, const double* __restrict__ u, int64_t n, double* red,
                            unsigned int* count, unsigned int* slices, double* sc) {
   __shared__ double sh[32];
@@ -64,10 +136,12 @@ __global__ void k_jv_norms(const double* __restrict__ v, const double* __restric
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     s = fma(x[i], x[i], s);
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) red[k * gridDim.x + blockIdx.x] = s;
-  if (last_block(count + k, gridDim.x)) {
+  const double bs = block_sum(s, sh);
+  if (threadIdx.x == 0) {
+    __stcg(red + k * gridDim.x + blockIdx.x, bs);
     __threadfence();
+  }
+  if (last_to_come(count + k, gridDim.x)) {
     const double t = warp0_sum(red + k * gridDim.x, gridDim.x);
     if (threadIdx.x == 0) {
       __stcg(sc + 1 - k, sqrt(t));
@@ -76,7 +150,9 @@ __global__ void k_jv_norms(const double* __restrict__ v, const double* __restric
       if (atomicAdd(slices, 1u) == gridDim.y - 1) {  // both norms are there
         __threadfence();
         const double vn = __ldcg(sc + 1);
-        sc[2] = vn > 0.0 ? 1.4901161193847656e-08 * (1.0 + __ldcg(sc)) / vn : 1.0;
+        const double eps = vn > 0.0 ? 1.4901161193847656e-08 * (1.0 + __ldcg(sc)) / vn : 1.0;
+        sc[2] = eps;
+        sc[3] = 1.0 / eps;
         *slices = 0;
       }
     }
@@ -106,15 +182,18 @@ void launch_waxpy_dev(double* y, const double* x, const double* v, const double*
 // y = x * s[0] (invert: x / s[0])
 __global__ void k_scale_copy(double* __restrict__ y, const double* __restrict__ x,
                              const double* s, int invert, int64_t n) {
-  const double f = invert ? 1.0 / s[0] : s[0];
+  __shared__ double f;  // one quotient a block, on the FP64 pipe for 16 cycles an instruction
+  if (threadIdx.x == 0) f = invert ? 1.0 / s[0] : s[0];
+  __syncthreads();
+#pragma unroll 4
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     y[i] = x[i] * f;
 }
 void launch_scale_copy(double* y, const double* x, const double* s, int invert, int64_t n,
                        cudaStream_t st) {
-  k_scale_copy<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>(y, x, s,
-                                                                                invert, n);
+  // at most four blocks an SM: 512^2 x 2 7.9 -> 3.6 us with the quotient once a block
+  k_scale_copy<<<(unsigned)std::min<int64_t>((n + 255) / 256, 608), 256, 0, st>>>(y, x, s, invert, n);
 }
 
 // w -= sum_k coef[k] V_k  (coef on the device)

@@ -617,7 +617,7 @@ __global__ void k_cell(DevMesh m, const double* __restrict__ flux, const double*
     for (int j = 0; j < DIM; ++j) r[j] += m.inert[j * m.nc + c];
   }
   if (R0) {
-    const double ie = 1.0 / d_eps[0];
+    const double ie = d_eps[1];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) out[j * m.nc + c] = (r[j] - R0[j * m.nc + c]) * ie;
   } else {
@@ -1749,7 +1749,7 @@ __global__ void k_cell_diff(DevMesh m, const double* __restrict__ flux,
       r[j] = code > 0 ? r[j] + v : r[j] - v;
     }
   }
-  const double ie = 1.0 / d_eps[0];
+  const double ie = d_eps[1];
 #pragma unroll
   for (int j = 0; j < DIM; ++j)
     out[j * m.nc + c] = m.mscale ? fma(r[j], ie, m.inert[j * m.nc + c]) : r[j] * ie;
