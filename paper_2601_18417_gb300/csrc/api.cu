@@ -1992,12 +1992,14 @@ static int rebuild_from_stencils(hofv_ctx* c) {
   invalidate_graphs(c);
   jv_invalidate(c);
   if (c->prec == HOFV_PREC_DF64) {
-    // the fits write the coefficients as doubles in their own order: clear
-    // the last tiles, whose slots past the last face or cell they leave alone
+    // the fits write the coefficients as doubles in their own order and leave
+    // alone what has none: slots past the last face or cell of a last tile and,
+    // in every tile, the weights of cell slots without a face (polygons,
+    // polyhedra), where the pairs' order has other cells' values
     const size_t ft = (size_t)c->S * kTile * c->Q * c->dim, ct = (size_t)c->S * kTile * c->nlf;
     if (c->nftile > 0)
       HOFV_CUDA(c, cudaMemsetAsync(c->d_fco + (c->nftile - 1) * ft, 0, sizeof(double) * ft, c->stream));
-    HOFV_CUDA(c, cudaMemsetAsync(c->d_cex + (c->nctile - 1) * ct, 0, sizeof(double) * ct, c->stream));
+    HOFV_CUDA(c, cudaMemsetAsync(c->d_cex, 0, sizeof(double) * ct * c->nctile, c->stream));
   }
   TRY(run_lsq(c));
   if (c->prec == HOFV_PREC_DF64)
