@@ -1238,6 +1238,8 @@ void launch_coef_format(double* a, int64_t chunks, int np, int rows, int to_df, 
 // shared memory as float pairs and are added in a fixed order.  Rows without
 // a flux (polygon and polyhedron slots past a cell's last face, traction
 // faces) are never read back and, where slots may be empty, load nothing.
+// A warp's slots past the last take its cell, with zero coefficients: a cell of
+// the stencil, so that a value that is not finite reaches no other cell by them.
 // Measured (us, one thread a (cell, face) -> this): 13^3 hexes p = 3 60 -> 25
 // (four warps a tile hide each other's latency), 48^3 hexes p = 3 187 -> 137
 // (0.55 of HBM: the gathers and the packed products), p = 2 148 -> 111, 512^2
@@ -1286,7 +1288,7 @@ __global__ void __launch_bounds__(UsShape<NLF>::THREADS, 512 / UsShape<NLF>::THR
   }
   int32_t id[U];
 #pragma unroll
-  for (int d = 0; d < U; ++d) id[d] = k + d * W < S ? __ldg(st + (k + d * W) * kTile) : 0;
+  for (int d = 0; d < U; ++d) id[d] = __ldg(st + min(k + d * W, S - 1) * kTile);
   for (int n0 = k; n0 < S; n0 += U * W) {
     float2 c[U][RPG], u[U][DIM];
 #pragma unroll
@@ -1301,10 +1303,7 @@ __global__ void __launch_bounds__(UsShape<NLF>::THREADS, 512 / UsShape<NLF>::THR
         u[d][j] = __ldg(reinterpret_cast<const float2*>(sw + (int64_t)id[d] * DIM + j));
     }
 #pragma unroll
-    for (int d = 0; d < U; ++d) {
-      const int n = n0 + (U + d) * W;
-      id[d] = n < S ? __ldg(st + n * kTile) : 0;
-    }
+    for (int d = 0; d < U; ++d) id[d] = __ldg(st + min(n0 + (U + d) * W, S - 1) * kTile);
 #pragma unroll
     for (int d = 0; d < U; ++d) {
 #pragma unroll
