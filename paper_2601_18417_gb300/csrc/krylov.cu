@@ -446,8 +446,10 @@ __global__ void k_cg_finish(int64_t nc, const T* __restrict__ invd, const T* __r
 //    memory, after one more block barrier; only the others' r, w and s go
 //    through L2, and only cells that another block reads are stored there
 //    (45^3 hexes, 30 iterations: 293 -> 272 us).
-//  * alpha needs no quotient of the previous alpha: beta gamma / alpha_prev =
-//    beta^2 (delta - ...)_prev, gamma / beta = gamma_prev.
+//  * In FP32 alpha needs no quotient of the previous alpha: beta gamma /
+//    alpha_prev = beta^2 (delta - ...)_prev, gamma / beta = gamma_prev; the
+//    scalars are doubles, so the roundings are far below the vectors'.  FP64
+//    keeps the quotients: 1 / gamma overflows where gamma is a subnormal number.
 // The sums keep their order (a warp's cells by shuffles in T, warps of 1024
 // cells in double, blocks in T), whatever the number of blocks.
 // ---------------------------------------------------------------------
@@ -561,8 +563,8 @@ __global__ void __launch_bounds__(kPersistThreads)
   const int64_t c0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t cstep = (int64_t)gridDim.x * blockDim.x;
   T pg[DIM], pd[DIM];  // per-thread partials in the vector precision
-  // threads j < DIM: 1 / gamma, denominator and alpha of the last iteration
-  double inv_gp = 0.0, den_p = 0.0, alpha_p = 0.0;
+  // threads j < DIM: 1 / gamma, gamma, denominator and alpha of the last iteration
+  double inv_gp = 0.0, gamma_p = 0.0, den_p = 0.0, alpha_p = 0.0;
   // the thread's cell (RES): its row of the matrix and its vectors; a
   // neighbour of the same block is an index into rs, another's is global
   constexpr bool ROW = RES && NLF <= 6;    // the row fits in registers
@@ -657,17 +659,24 @@ __global__ void __launch_bounds__(kPersistThreads)
     if (threadIdx.x < DIM) {
       const int j = threadIdx.x;
       const double gamma = s_sum[2 * j], delta = s_sum[2 * j + 1];
-      const double beta = gamma * inv_gp;  // 0 in the first iteration
-      const double den = it == 0 ? delta : alpha_p != 0.0 ? fma(-(beta * beta), den_p, delta) : 0.0;
+      double beta, den;
+      if constexpr (sizeof(T) == 8) {  // the quotients themselves
+        beta = gamma_p != 0.0 ? gamma / gamma_p : 0.0;  // 0 in the first iteration
+        den = it == 0 ? delta : alpha_p != 0.0 ? delta - beta * gamma / alpha_p : 0.0;
+        gamma_p = gamma;
+      } else {
+        beta = gamma * inv_gp;
+        den = it == 0 ? delta : alpha_p != 0.0 ? fma(-(beta * beta), den_p, delta) : 0.0;
+        den_p = den;
+      }
       const double alpha = den != 0.0 ? gamma / den : 0.0;
-      den_p = den;
       alpha_p = alpha;
       s_ab[j] = (T)alpha;
       s_ab[DIM + j] = (T)beta;
     }
     __syncthreads();
     // the next beta's divisor, while the other warps go on
-    if (threadIdx.x < DIM) {
+    if (sizeof(T) == 4 && threadIdx.x < DIM) {
       const double gamma = s_sum[2 * threadIdx.x];
       inv_gp = gamma != 0.0 ? 1.0 / gamma : 0.0;
     }
