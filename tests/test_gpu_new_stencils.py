@@ -18,7 +18,8 @@ def test_the_same_stencils_give_the_same_coefficients(name):
     pb, ctx = _make(name)
     lay = ctx.layout
     nf = lay.n_internal + lay.n_disp
-    empty = pb.orc.cell_faces() < 0
+    sides = (pb.orc.cell_faces() >= 0).sum(axis=1)
+    empty = np.arange(ctx.faces_per_cell)[None, :] >= sides[:, None]
     assert empty.any() == (name != "quad-q2")
     ctx.set_precision(hofv.PREC_DF64)
     st, co = ctx.get_face_data(0, nf)
