@@ -568,9 +568,12 @@ int hofv_mg_info(hofv_ctx* ctx, int32_t* levels, int64_t* sizes, int32_t max_siz
 /* Self-test of the bounded waits: the approximate-Jacobian solve runs as one
    cooperative launch whose blocks meet at grid barriers; each wait gives up
    after a bounded number of polls, latches an error flag and returns, and
-   the host reports HOFV_ECUDA at its next synchronisation.  This launches
-   two blocks that wait for a third arrival that never comes; on return
-   *timed_out (HOST) is 1 when the wait ran out and was latched, and the
+   the host reports HOFV_ECUDA at its next synchronisation; until then later
+   solves on the stream return without waiting.  This launches
+   two blocks that wait for a third arrival that never comes, and behind them
+   two whose arrivals are already counted; on return
+   *timed_out (HOST) is 1 when the wait ran out and was latched and neither
+   launch passed its barrier, and the
    flag has been cleared so the context stays usable.  Synchronises. */
 int hofv_selftest_barrier(hofv_ctx* ctx, int32_t* timed_out);
 

@@ -461,24 +461,33 @@ struct GridBarrier {
   int* err;
 };
 
+// Whether an earlier launch's wait ran out and the host has not cleared the
+// flag yet: its counters are then not those of a new launch.  Thread 0 reads
+// it when the kernel begins and hands it to the barriers.
+__device__ __forceinline__ bool barrier_failed(const GridBarrier& gb) {
+  return threadIdx.x == 0 && *(volatile int*)gb.err != 0;
+}
+
 // Arrive, and wait until `target` arrivals have been counted since the
 // launch began.  Returns false (the same for the whole block) when the wait
-// ran out or another block's did.
-__device__ __forceinline__ bool grid_barrier(const GridBarrier& gb, unsigned int target,
+// ran out, another block's did, or an earlier launch's had (failed).
+__device__ __forceinline__ bool grid_barrier(const GridBarrier& gb, unsigned int target, bool failed,
                                              unsigned int spin_limit = kBarrierSpinLimit) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(gb.count, 1u);
-    int ok = 1;
-    unsigned int spins = 0, now;
-    for (;;) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(gb.count) : "memory");
-      if (now >= target) break;
-      if (++spins > spin_limit || ((spins & 1023u) == 0 && *(volatile int*)gb.err)) {
-        ok = 0;
-        break;
+    int ok = !failed;
+    if (ok) {
+      __threadfence();
+      atomicAdd(gb.count, 1u);
+      unsigned int spins = 0, now;
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(gb.count) : "memory");
+        if (now >= target) break;
+        if (++spins > spin_limit || ((spins & 1023u) == 0 && *(volatile int*)gb.err)) {
+          ok = 0;
+          break;
+        }
       }
     }
     if (!ok) atomicExch(gb.err, 1);
@@ -553,6 +562,7 @@ __global__ void __launch_bounds__(kPersistThreads)
   __shared__ double s_sum[NS];
   __shared__ T s_ab[2 * DIM];              // alpha, beta in the vector precision
   const unsigned int nb = gridDim.x;
+  const bool failed = nb > 1 && barrier_failed(gb);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t nv = CV::N * nc;
   T* r[2] = {rwork, rwork + nv};
@@ -646,7 +656,7 @@ __global__ void __launch_bounds__(kPersistThreads)
     if (nb == 1) {
       __syncthreads();
     } else {
-      if (!grid_barrier(gb, (unsigned int)(it + 1) * nb)) return;
+      if (!grid_barrier(gb, (unsigned int)(it + 1) * nb, failed)) return;
       if (wid < NS) {  // every block forms the same sums in the same order
         T t = (T)0;
 #pragma unroll 5
@@ -887,24 +897,32 @@ static void cg_run(hofv_ctx* c, const T* diag, const T* invd, const T* off, T* w
                                                                      p, sc, zout);
 }
 
-// Two co-resident blocks wait at a barrier that expects one more arrival
-// than exists: the wait must run out and latch the error flag.
-__global__ void k_barrier_probe(GridBarrier gb, unsigned int spin_limit) {
-  grid_barrier(gb, gridDim.x + 1, spin_limit);  // the count stays: the host clears it
+// Two co-resident blocks at a barrier.  With extra = 1 it expects one more
+// arrival than exists: the wait must run out and latch the error flag.
+__global__ void k_barrier_probe(GridBarrier gb, unsigned int extra, unsigned int spin_limit, unsigned int* passed) {
+  const bool failed = barrier_failed(gb);
+  // the count stays: the host clears it
+  if (grid_barrier(gb, gridDim.x + extra, failed, spin_limit) && threadIdx.x == 0) atomicExch(passed, 1u);
 }
 
+// A wait that runs out, and behind it, before the host looks, a launch whose
+// arrivals are already counted: neither may pass.
 int barrier_selftest(hofv_ctx* c, int* timed_out) {
   *timed_out = 0;
   if (!c->d_bar) return fail(c, HOFV_ESTATE, "hofv_build_stencils must come first");
   GridBarrier gb{c->d_bar, c->d_bar + 1, reinterpret_cast<int*>(c->d_bar + 2)};
-  unsigned int limit = 1u << 14;
-  void* args[] = {&gb, &limit};
-  HOFV_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_barrier_probe, dim3(2), dim3(32), args,
-                                           0, c->stream));
+  unsigned int limit = 1u << 14, extra;
+  unsigned int* passed = c->d_bar + 3;
+  void* args[] = {&gb, &extra, &limit, &passed};
+  for (unsigned int e : {1u, 0u}) {
+    extra = e;
+    HOFV_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_barrier_probe, dim3(2), dim3(32), args, 0,
+                                             c->stream));
+  }
   HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
-  int err = 0;
-  HOFV_CUDA(c, cudaMemcpy(&err, c->d_bar + 2, sizeof(int), cudaMemcpyDeviceToHost));
-  *timed_out = err != 0;
+  int flags[2] = {0, 0};  // the error flag, and `passed`
+  HOFV_CUDA(c, cudaMemcpy(flags, c->d_bar + 2, sizeof(flags), cudaMemcpyDeviceToHost));
+  *timed_out = flags[0] != 0 && flags[1] == 0;
   HOFV_CUDA(c, cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)));
   return 0;
 }
