@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "fixed_point.cuh"
 #include "hofv_internal.cuh"
 
 namespace hofv {
@@ -59,9 +60,6 @@ namespace hofv {
 // Rows and stencils whose largest binade lies outside [kFxMin, kFxMax] (tiny,
 // huge, infinite or NaN values) are summed by FP64 FMAs.
 // ---------------------------------------------------------------------
-constexpr int kFxMin = 540, kFxMax = 1560;  // biased exponents: the scales stay normal numbers
-constexpr uint16_t kFxPlain = 0xffff;       // row exponent of a row to be summed by FMAs
-
 // largest biased exponent of each coefficient row of [tile][S][cs]
 __global__ void k_row_exponents(const double* __restrict__ a, int S, int cs, int64_t n,
                                 uint16_t* __restrict__ out) {
@@ -82,47 +80,6 @@ void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_
   const int64_t n = tiles * cs;
   if (n > 0) k_row_exponents<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, S, cs, n, out);
 }
-
-// |c| 2^(1078 - E) truncated, below 2^56, as 28-bit limbs (hi, lo) with c's sign
-__device__ __forceinline__ int2 fx_coef(double c, int E) {
-  const int h = __double2hiint(c);
-  const uint32_t l = (uint32_t)__double2loint(c);
-  const int sh = min(E - ((h >> 20) & 0x7ff), 55);  // 55 for zero: kFxMin
-  // the significand at the top of 64 bits
-  const uint32_t mh = __funnelshift_l(l, (uint32_t)h, 11) | 0x80000000u;
-  const uint64_t m = (uint64_t)mh << 32 | (l << 11);
-  uint32_t hi;  // a shift by 32 and more gives zero
-  asm("shr.u32 %0, %1, %2;" : "=r"(hi) : "r"(mh), "r"(sh + 4));
-  const int lo = (int)((uint32_t)(m >> (sh + 8)) & 0xfffffffu);
-  return h < 0 ? make_int2(-(int)hi, -lo) : make_int2((int)hi, lo);
-}
-
-// u 2^(1077 - E) rounded, at most 2^55, as 28-bit limbs (hi, lo), the low one
-// in [-2^27, 2^27)
-__device__ __forceinline__ int2 fx_value(int h, int l, int E) {
-  const int sh = min(E - ((h >> 20) & 0x7ff), 63);  // 63 for zero
-  const uint64_t mant = (uint64_t)(uint32_t)((h & 0xfffff) | 0x100000) << 32 | (uint32_t)l;
-  int64_t v = (int64_t)((((mant << 3) >> sh) + 1) >> 1);
-  if (h < 0) v = -v;
-  const int64_t hi = (v + (1 << 27)) >> 28;
-  return make_int2((int)hi, (int)((uint32_t)v - ((uint32_t)hi << 28)));
-}
-
-// t in units of 2^56 2^(Ec - 1078 + Eu - 1077)
-__device__ __forceinline__ double fx_scale(int64_t t, int Ec, int Eu) {
-  return (double)t * __hiloint2double((1023 + Ec + Eu - 2099) << 20, 0);
-}
-
-// sums of products of one component: the high limbs' (2^56) and the mixed (2^28)
-struct FxSum {
-  int64_t hh = 0, x = 0;
-  __device__ __forceinline__ void mac(int2 q, int uh, int ul) {
-    hh += (int64_t)q.x * uh;
-    x += (int64_t)q.x * ul;
-    x += (int64_t)q.y * uh;
-  }
-  __device__ __forceinline__ int64_t total() const { return hh + ((x + (1 << 27)) >> 28); }
-};
 
 // The values at the stencils of `items` consecutive faces or cells (item0 the
 // first) as limbs in shared memory, ua[n * STRIDE + k] components 0 and 1 and
@@ -190,11 +147,12 @@ __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, cons
     if (fx)
       for (int n = s0; n < S; n += step) {  // a thread converts what it stored
         const int4 a = ua[n * stride + k];
-        const int2 x = fx_value(a.x, a.y, E[0]), y = fx_value(a.z, a.w, E[1]);
-        ua[n * stride + k] = make_int4(x.x, x.y, y.x, y.y);
+        const FxLimbs x = fx_value(a.x, a.y, E[0]), y = fx_value(a.z, a.w, E[1]);
+        ua[n * stride + k] = make_int4(x.hi, x.lo, y.hi, y.lo);
         if constexpr (DIM == 3) {
           const int2 b = ub[n * stride + k];
-          ub[n * stride + k] = fx_value(b.x, b.y, E[2]);
+          const FxLimbs z = fx_value(b.x, b.y, E[2]);
+          ub[n * stride + k] = make_int2(z.hi, z.lo);
         }
       }
   }
@@ -218,7 +176,7 @@ struct FxRow {
     for (; n0 + 2 * K <= S; n0 += K) {  // every request in range
 #pragma unroll
       for (int d = 0; d < K; ++d) {
-        const int2 q = fx_coef(c[d], E);
+        const FxLimbs q = fx_coef(c[d], E);
         c[d] = __ldg(co + d * CS);
         mac(q, n0, d);
       }
@@ -226,7 +184,7 @@ struct FxRow {
     }
 #pragma unroll
     for (int d = 0; d < K; ++d) {
-      const int2 q = fx_coef(c[d], E);
+      const FxLimbs q = fx_coef(c[d], E);
       if (n0 + K + d < S) c[d] = __ldg(co + d * CS);
       if (n0 + d < S) mac(q, n0, d);
     }
@@ -242,7 +200,7 @@ struct FxAll {
   const int4* ua;
   const int2* ub;
   FxSum s[DIM];
-  __device__ __forceinline__ void operator()(int2 q, int n0, int d) {
+  __device__ __forceinline__ void operator()(FxLimbs q, int n0, int d) {
     const int4 a = ua[n0 * STRIDE + d * STRIDE];
     s[0].mac(q, a.x, a.y);
     s[1].mac(q, a.z, a.w);
