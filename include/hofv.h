@@ -67,7 +67,7 @@ extern "C" {
 #define HOFV_PC_NEJ 4    /* near-exact Jacobian (linear law), inner GMRES with AJMG */
 
 /* arithmetic of the gradient contraction (hofv_set_precision) */
-#define HOFV_PREC_FP64 0   /* FP64 operands, sums in fixed point (default) */
+#define HOFV_PREC_FP64 0   /* FP64 operands and sums, in fixed point where exact (default) */
 #define HOFV_PREC_DF64 1   /* double-float pairs on the FP32 pipe, everything else FP64 */
 
 /* point sets for hofv_get_points */
@@ -297,11 +297,13 @@ int hofv_set_contraction(hofv_ctx* ctx, int on);
    reconstruction coefficients with the stencil values (the displacement
    gradient at every face Gauss point, eq. faceQuadGrad, and the
    extrapolated face values of the stabilisation, eq. alphaJump).
-   HOFV_PREC_FP64 (default) takes FP64 coefficients and values and sums their
-   products in 64-bit fixed point: each slot's error is at most 2^-53 of the
-   row's largest coefficient times the stencil's largest value, where FP64
-   fused multiply-adds round at 2^-53 of every partial sum (they are used where
-   either is not finite or beyond about 1e+-145).  HOFV_PREC_DF64 stores
+   HOFV_PREC_FP64 (default) takes FP64 coefficients and values.  Where a row's
+   first products are large enough against its largest coefficient times the
+   stencil's largest value, their sum is formed in 64-bit fixed point and
+   rounded once, which leaves a smaller error than FP64 fused multiply-adds
+   (a tenth on smooth fields); elsewhere (values that differ by orders of
+   magnitude within a stencil, or are not finite or beyond about 1e+-140) the
+   products are summed by FP64 fused multiply-adds.  HOFV_PREC_DF64 stores
    each coefficient as a pair of floats (hi, lo), hi + lo its value
    rounded to 48 significant bits, splits the state exactly into three
    floats, and forms each product exactly (TwoProduct by FMA, Dekker 1971)

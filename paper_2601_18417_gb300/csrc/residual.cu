@@ -19,8 +19,8 @@
 //   k_cell_avg : inertia term of the BDF2 dynamics, only when enabled
 //
 // Operands and results are FP64; the contractions over the stencils are formed
-// in fixed point (more exact than FP64 FMAs, and not bound by their rate) or,
-// on request, in double-float arithmetic.  A tile's (face, row) pairs are laid
+// in fixed point where that is as exact as FP64 FMAs, whose rate does not bound
+// it, by those FMAs elsewhere or, on request, in double-float arithmetic.  A tile's (face, row) pairs are laid
 // out so that consecutive threads own consecutive coefficient rows.
 #include <algorithm>
 #include <type_traits>
@@ -32,35 +32,55 @@ namespace hofv {
 
 // ---------------------------------------------------------------------
 // Fixed-point contraction of FP64 coefficients with FP64 values (the
-// arithmetic of HOFV_PREC_FP64).
+// arithmetic of HOFV_PREC_FP64; fixed_point.cuh).
 //
 // GB300 issues 2 FP64 FMAs a clock and SM, a fraction of what one coefficient
 // a product needs at HBM speed, but many times that of 32 x 32 -> 64 bit
 // integer multiply-adds.  So a sum sum_N c_N u_N is formed exactly but for
-// the representation of its operands: the coefficients of a row in units of
-// 2^-56 of the row's largest binade (truncated, 56 bits), the values of a
-// stencil in units of 2^-55 of its largest (rounded, 55 bits), each as two
-// 28-bit limbs; the products of the high limbs and of the high with the low
-// ones are summed without rounding in 64 bits.  Left out are the products of
-// the low limbs (zero on average, the value's low limb being signed).  The
-// bounds |C1|, |C0| < 2^28, |U1|, |U0| <= 2^27 and kMaxS = 128 slots keep both
-// sums below 2^63.  A sum of FP64 FMAs rounds at 2^-53 of each partial sum, so
-// this is the more accurate of the two.
+// the representation of its operands: the coefficients of a row as integers
+// of 59 bits in units of 2^-59 of a power of two 2^e, the values of a stencil
+// as integers of 55 bits in units of 2^-55 of their largest binade, both rounded
+// and each as two limbs; the products of the high limbs and of the high with
+// the low ones are summed without rounding in 64 bits, and the sum is rounded
+// once.  Left out are the products of the low limbs (zero on average, the value's
+// low limb being signed).  2^e is above each coefficient, and sum |c_N| <= 15 2^e;
+// with that, |U1| <= 2^27, |U0| <= 2^27, |C0| <= 2^28 and kMaxS = 128 slots both sums
+// stay below 2^63.
 //
-// What bounds it: integer issue.  A coefficient takes about 15 instructions to
+// The error of that scales with the largest coefficient times the largest value,
+// the error of FMAs with the partial sums.  Where the products are all small
+// against those maxima (one value among zeros, a far cell's large value, a
+// field falling by ten a cell) FMAs are the more accurate, and they are taken
+// then: a row's sum is left in fixed point only if its first products add up to
+// 2^-4 (2-D) or 2^-5 (3-D) of 2^e times the values' binade (fx_sure).
+// Errors of this rule and of FMAs alone over sum |c_N u_N|, rms over the gradient
+// rows of jittered p = 3 hexes (quads), and the rows left in fixed point:
+//   smooth field         1.7e-17 and 1.5e-16 (1.3e-17 and 5.6e-17)   all
+//   random values        1.8e-17 and 1.3e-16 (3.4e-17 and 1.1e-16)   all (99 %)
+//   zero across the face 2.0e-17 and 1.6e-16 (3.2e-17 and 1.2e-16)   99.9 % (98.9 %)
+//   falling by e a cell  4.2e-17 and 9.2e-17 (4.1e-17 and 6.1e-17)   99.9 % (85 %)
+//   falling by 10 a cell 8.7e-17 and 1.0e-16 (5.7e-17 and 6.5e-17)   19 % (8 %)
+//   one value            4.6e-17 and 4.6e-17 (4.7e-17 and 4.7e-17)   12 % (9 %)
+//
+// What bounds it: integer issue.  A coefficient takes about 17 instructions to
 // split and, for three components, nine multiply-adds at 32 a clock and SM (209
-// of the 467 us on 32^3 hexes; the bytes take 257).  Measured, FP64 FMAs -> this
-// (us): k_flux 32^3 hexes p = 3 neo-Hookean 1427 -> 467 (the FMAs alone bound it
-// at 1140), 40^3 p = 2 1074 -> 353, 2 255^2 triangles 107 -> 68, 20-layer prisms
-// 1107 -> 397, 6 17^3 tetrahedra 268 -> 116; k_ustar 32^3 hexes 102 -> 59, 512^2
-// quads 78 -> 57.  Strides known to the compiler and a loop without range checks
-// gave 666 -> 497 of that, the significand taken from the top of its word 478.
-// Not kept: every 5th slot by FP64 FMAs beside the others (515), two of five (682).
+// of the 499 us on 32^3 hexes; the bytes take 257).  Measured on smooth fields,
+// FP64 FMAs alone -> this (us): k_flux 32^3 hexes p = 3 neo-Hookean 1427 -> 499,
+// 40^3 p = 2 1077 -> 380, 2 255^2 triangles 110 -> 78, 20-layer prisms 1104 -> 420,
+// 6 17^3 tetrahedra 272 -> 136; k_ustar 32^3 hexes 107 -> 70, 40^3 148 -> 101, 512^2
+// quads 83 -> 67.  Without the check and the way to FMAs the same rows took 476,
+// 355, 76, 390, 119, 65, 97 and 65, the tetrahedra among them because 0.1 % of their
+// rows go that way.  A state that takes nearly all rows there (values spread
+// over 2^40): k_flux 1322, 934, 137, 981, 293, k_ustar 119, 175, 107.  Strides known to the
+// compiler and a loop without range checks gave 666 -> 497 of the first.  Not
+// kept: every 5th slot by FP64 FMAs beside the others (515 for 467), two of five
+// (682); the FMAs behind a barrier (516 for 499) or inlined (504); the limbs cut from
+// one 64-bit integer (684).
 //
 // Rows and stencils whose largest binade lies outside [kFxMin, kFxMax] (tiny,
-// huge, infinite or NaN values) are summed by FP64 FMAs.
+// huge, infinite or NaN values) are summed by FP64 FMAs too.
 // ---------------------------------------------------------------------
-// largest biased exponent of each coefficient row of [tile][S][cs]
+// the exponent that scales each coefficient row of [tile][S][cs]
 __global__ void k_row_exponents(const double* __restrict__ a, int S, int cs, int64_t n,
                                 uint16_t* __restrict__ out) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (tile, row)
@@ -68,12 +88,14 @@ __global__ void k_row_exponents(const double* __restrict__ a, int S, int cs, int
   const double* __restrict__ p = a + e / cs * S * cs + e % cs;
   int mx = 0;
   bool zero = true;
+  double sum = 0.0;
   for (int k = 0; k < S; ++k) {
     const double v = p[(int64_t)k * cs];
     zero &= v == 0.0;
     mx = max(mx, (__double2hiint(v) >> 20) & 0x7ff);
+    sum += fabs(v);
   }
-  out[e] = zero ? (uint16_t)kFxMin : mx < kFxMin || mx > kFxMax ? kFxPlain : (uint16_t)mx;
+  out[e] = fx_row_exponent(mx, zero, sum);
 }
 
 void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_t* out, cudaStream_t st) {
@@ -134,8 +156,9 @@ __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, cons
 #pragma unroll
     for (int j = 0; j < DIM; ++j) {
       const int key = ex[k * DIM + j];
-      E[j] = key == 0 ? kFxMin : key >> 20;  // all zero: any scale
-      fx &= E[j] >= kFxMin && E[j] <= kFxMax;
+      E[j] = key >> 20;
+      fx &= key == 0 || (E[j] >= kFxMin && E[j] <= kFxMax);
+      if (key == 0) E[j] = kFxZero;
     }
   }
   __syncthreads();
@@ -159,20 +182,30 @@ __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, cons
   __syncthreads();
 }
 
-// Streams the S coefficients of the row co (CS between slots) as limbs to
-// mac(limbs, n0, d), slot n0 + d; E is the row's exponent.  K slots are requested
-// ahead in registers (begin, before the values are ready).
-template <int K, int CS>
+// Streams the S coefficients of the row co (CS between slots) as limbs, the
+// first HEAD to mac.head(limbs, n), those from n0 on to mac(limbs, n0, d),
+// slot n0 + d; E is the row's exponent.  K slots are requested ahead in registers
+// (begin, before the values are ready).
+template <int K, int CS, int HEAD>
 struct FxRow {
+  static_assert(HEAD % K == 0, "the head takes whole rounds of requests");
   double c[K];
   __device__ __forceinline__ void begin(const double* __restrict__ co, int S) {
 #pragma unroll
     for (int d = 0; d < K; ++d) c[d] = d < S ? __ldg(co + d * CS) : 0.0;
   }
   template <typename F>
-  __device__ __forceinline__ void run(const double* __restrict__ co, int S, int E, F&& mac) {
-    int n0 = 0;
-    co += K * CS;
+  __device__ __forceinline__ void head(const double* __restrict__ co, int S, int E, F& mac) {
+#pragma unroll
+    for (int n = 0; n < HEAD; ++n) {
+      const FxLimbs q = fx_coef(c[n % K], E);
+      if (n + K < S) c[n % K] = __ldg(co + (n + K) * CS);
+      if (n < S) mac.head(q, n);
+    }
+  }
+  template <typename F>
+  __device__ __forceinline__ void tail(const double* __restrict__ co, int n0, int S, int E, F& mac) {
+    co += (n0 + K) * CS;
     for (; n0 + 2 * K <= S; n0 += K) {  // every request in range
 #pragma unroll
       for (int d = 0; d < K; ++d) {
@@ -200,6 +233,7 @@ struct FxAll {
   const int4* ua;
   const int2* ub;
   FxSum s[DIM];
+  uint32_t size[DIM];
   __device__ __forceinline__ void operator()(FxLimbs q, int n0, int d) {
     const int4 a = ua[n0 * STRIDE + d * STRIDE];
     s[0].mac(q, a.x, a.y);
@@ -209,24 +243,60 @@ struct FxAll {
       s[2].mac(q, b.x, b.y);
     }
   }
+  __device__ __forceinline__ void head(FxLimbs q, int n) {
+    (*this)(q, n, 0);
+    const int4 a = ua[n * STRIDE];
+    size[0] += fx_size(q, a.x);
+    size[1] += fx_size(q, a.z);
+    if constexpr (DIM == 3) size[2] += fx_size(q, ub[n * STRIDE].x);
+  }
+  // the sums are exact enough, or all coefficients (exponent E) or values
+  // (exponents ex) are zero
+  __device__ __forceinline__ bool sure(int E, const int* ex) const {
+    bool r = true;
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) r &= size[j] >= fx_sure(DIM) || ex[j] == kFxZero;
+    return r || E == kFxZero;
+  }
 };
 
-// the same sum by FP64 FMAs
+// the same sum by FP64 FMAs, SL slots CS apart, U slots' requests at a time
 template <int DIM>
-__device__ __noinline__ void plain_row(const double* __restrict__ co, int64_t cs, int SL,
-                                       const int32_t* __restrict__ st, const double* __restrict__ w,
-                                       int64_t ws, double* acc) {
-  double s[DIM];
+struct PlainSum {
+  double v[DIM];
+};
+template <int DIM, int CS>
+__device__ __noinline__ PlainSum<DIM> plain_row(const double* __restrict__ co, int SL,
+                                                const int32_t* __restrict__ st,
+                                                const double* __restrict__ w, int64_t ws) {
+  constexpr int U = DIM == 2 ? 5 : 4;
+  PlainSum<DIM> s;
 #pragma unroll
-  for (int j = 0; j < DIM; ++j) s[j] = 0.0;
-  for (int n = 0; n < SL; ++n) {
-    const int32_t id = __ldg(st + n * kTile);
-    const double c = __ldg(co + n * cs);
+  for (int j = 0; j < DIM; ++j) s.v[j] = 0.0;
+  int n = 0;
+  for (; n + U <= SL; n += U) {
+    int32_t id[U];
+    double c[U], u[U][DIM];
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) s[j] = fma(c, __ldg(w + j * ws + id), s[j]);
+    for (int d = 0; d < U; ++d) id[d] = __ldg(st + (n + d) * kTile);
+#pragma unroll
+    for (int d = 0; d < U; ++d) {
+      c[d] = __ldg(co + (int64_t)(n + d) * CS);
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) u[d][j] = __ldg(w + j * ws + id[d]);
+    }
+#pragma unroll
+    for (int d = 0; d < U; ++d)
+#pragma unroll
+      for (int j = 0; j < DIM; ++j) s.v[j] = fma(c[d], u[d][j], s.v[j]);
   }
+  for (; n < SL; ++n) {
+    const int32_t id = __ldg(st + n * kTile);
+    const double c = __ldg(co + (int64_t)n * CS);
 #pragma unroll
-  for (int j = 0; j < DIM; ++j) acc[j] = s[j];
+    for (int j = 0; j < DIM; ++j) s.v[j] = fma(c, __ldg(w + j * ws + id), s.v[j]);
+  }
+  return s;
 }
 
 // shared memory of the limbs of a number of items
@@ -246,11 +316,15 @@ struct UstarShape {
   // SM with threads: fewer cells a block, more threads a row
   static constexpr int CPB = DIM == 2 ? 32 : 16;
   static constexpr int ROWS = CPB * NLF;
-  // four threads a row: 32^3 hexes 73 -> 59 us; two on 512^2 quads 57 -> 71
+  // four threads a row: 32^3 hexes 73 -> 59 us; two on 512^2 quads 57 -> 71 (both
+  // before the sums were checked, 70 and 67 now)
   static constexpr int W = NLF >= 8 || DIM == 2 ? 1 : 4;
   static constexpr int THREADS = ROWS * W;
   static constexpr int BLOCKS = 1152 / THREADS;
-  static size_t smem(int S) { return fx_smem_bytes<DIM>(S, CPB) + sizeof(int64_t) * (W - 1) * ROWS * DIM; }
+  // the parts' sums: FxTotal's h and l, or a double in h's place
+  static size_t smem(int S) {
+    return fx_smem_bytes<DIM>(S, CPB) + (sizeof(int64_t) + sizeof(uint32_t)) * (W - 1) * ROWS * DIM;
+  }
 };
 
 template <int DIM, int NLF>
@@ -260,10 +334,12 @@ __global__ void __launch_bounds__(UstarShape<DIM, NLF>::THREADS, UstarShape<DIM,
   constexpr int CPB = SH::CPB, ROWS = SH::ROWS, W = SH::W, CS = kTile * NLF;
   extern __shared__ __align__(16) double sm[];
   __shared__ int ex[CPB * DIM];
+  __shared__ uint8_t sure[W > 1 ? ROWS : 1];  // FxAll::sure of the row's first part
   const int S = m.S;
   int4* ua = reinterpret_cast<int4*>(sm);                                        // [S][CPB]
   int2* ub = reinterpret_cast<int2*>(ua + S * CPB);                              // [S][CPB]
   int64_t* part = reinterpret_cast<int64_t*>(ub + (DIM == 3 ? S * CPB : 0));     // [W-1][DIM][ROWS]
+  uint32_t* part_l = reinterpret_cast<uint32_t*>(part + (W - 1) * ROWS * DIM);   // the same
   const int64_t cell0 = (int64_t)blockIdx.x * CPB;
   const int it = threadIdx.x % ROWS, p = threadIdx.x / ROWS;
   const int ci = it / NLF, lf = it % NLF;
@@ -271,41 +347,69 @@ __global__ void __launch_bounds__(UstarShape<DIM, NLF>::THREADS, UstarShape<DIM,
   const bool on = cell < m.nc;
   const int row = (int)(cell % kTile) * NLF + lf;
   const int n0 = p * S / W, len = (p + 1) * S / W - n0;  // this thread's slots
-  const double* __restrict__ co = m.cex + tile * (int64_t)S * CS + row;
-  FxRow<5, CS> r;
-  r.begin(co + (int64_t)n0 * CS, on ? len : 0);
+  const double* __restrict__ co = m.cex + tile * (int64_t)S * CS + row + (int64_t)n0 * CS;
+  constexpr int HEAD = 10;
+  FxRow<5, CS, HEAD> r;
+  r.begin(co, on ? len : 0);
   const int E = on ? m.cexp[tile * CS + row] : kFxPlain;
   const int64_t ws = m.wst;  // stride of the state read
   fx_gather<DIM, SH::THREADS, CPB>(m.cst, w, ws, S, cell0, (int)min((int64_t)CPB, m.nc - cell0), ua, ub, ex);
-  const bool fx = E != kFxPlain && ex[ci * DIM] != 0;
-  int64_t t[DIM];
+  bool fx = E != kFxPlain && ex[ci * DIM] != 0;
+  FxTotal t[DIM];
   if (fx) {
-    FxAll<DIM, CPB> a{ua + n0 * CPB + ci, ub + n0 * CPB + ci, {}};
-    r.run(co + (int64_t)n0 * CS, len, E, a);
+    FxAll<DIM, CPB> a{ua + n0 * CPB + ci, ub + n0 * CPB + ci, {}, {}};
+    if (p == 0) {
+      r.head(co, len, E, a);
+      const bool ok = a.sure(E, ex + ci * DIM);
+      if (W == 1) fx = ok;
+      else sure[it] = ok;
+    }
+    if (fx) r.tail(co, p == 0 ? HEAD : 0, len, E, a);
 #pragma unroll
     for (int j = 0; j < DIM; ++j) t[j] = a.s[j].total();
-  }
-  if (W > 1) {
-    if (fx && p > 0) {
+    if (W > 1 && p > 0) {
 #pragma unroll
-      for (int j = 0; j < DIM; ++j) part[((p - 1) * DIM + j) * ROWS + it] = t[j];
+      for (int j = 0; j < DIM; ++j) {
+        part[((p - 1) * DIM + j) * ROWS + it] = t[j].h;
+        part_l[((p - 1) * DIM + j) * ROWS + it] = t[j].l;
+      }
     }
+  }
+  bool again = !fx;  // some row of the block is to be summed by FMAs
+  if (W > 1) {
     __syncthreads();
+    fx = fx && sure[it];
+    again = __syncthreads_or(on && !fx);
+  }
+  PlainSum<DIM> acc;
+  if (again) {
+    if (on && !fx)
+      acc = plain_row<DIM, CS>(co, len, m.cst + tile * (int64_t)S * kTile + n0 * kTile + cell % kTile, w, ws);
+    if (W > 1) {
+      if (on && !fx && p > 0) {
+#pragma unroll
+        for (int j = 0; j < DIM; ++j)
+          part[((p - 1) * DIM + j) * ROWS + it] = __double_as_longlong(acc.v[j]);
+      }
+      __syncthreads();
+    }
   }
   if (!on || p > 0) return;
-  double acc[DIM];
-  if (fx) {
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) {
+  for (int j = 0; j < DIM; ++j) {
+    if (fx) {
 #pragma unroll
-      for (int k = 0; k < W - 1; ++k) t[j] += part[(k * DIM + j) * ROWS + it];
-      acc[j] = fx_scale(t[j], E, ex[ci * DIM + j]);
+      for (int k = 0; k < W - 1; ++k) {
+        t[j].h += part[(k * DIM + j) * ROWS + it];
+        t[j].l += part_l[(k * DIM + j) * ROWS + it];
+      }
+      acc.v[j] = fx_scale(t[j], E, ex[ci * DIM + j]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < W - 1; ++k) acc.v[j] += __longlong_as_double(part[(k * DIM + j) * ROWS + it]);
     }
-  } else {
-    plain_row<DIM>(co, CS, S, m.cst + tile * (int64_t)S * kTile + cell % kTile, w, ws, acc);
+    ustar[(cell * NLF + lf) * DIM + j] = w[j * ws + cell] + acc.v[j];
   }
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) ustar[(cell * NLF + lf) * DIM + j] = w[j * ws + cell] + acc[j];
 }
 
 // ---------------------------------------------------------------------
@@ -450,7 +554,7 @@ __device__ __forceinline__ void traction(const double (&G)[3][3], const double* 
 // ---------------------------------------------------------------------
 // Blocks of 192 threads at most: 467 us against 478 with 384 (32^3 hexes p = 3),
 // 353 against 372 (40^3 p = 2), as more blocks mix their phases; 1152 threads an
-// SM: 478 against 537 with 768.
+// SM: 478 against 537 with 768 (all before the sums were checked).
 template <int DIM, int Q>
 struct FluxShape {
   static constexpr int R = Q * DIM;  // rows a face, at most 96 (8 fan slots of 2 x 2 points)
@@ -487,7 +591,10 @@ __global__ void __launch_bounds__(FluxShape<DIM, Q>::THREADS, FluxShape<DIM, Q>:
     // corner) are neither read nor formed
     const bool live = fi < nf && (m.fql == nullptr || r < __ldg(m.fql + f) * DIM);
     const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + row;
-    FxRow<5, kTile * R> rw;
+    // slots that are checked: the nearest ring of cells (with 10 on tetrahedra one
+    // warp in twelve went on to FMAs)
+    constexpr int HEAD = DIM == 2 ? 10 : 15;
+    FxRow<5, kTile * R, HEAD> rw;
     rw.begin(co, live ? S : 0);
     const int E = live ? m.fexp[tile * kTile * R + row] : kFxPlain;
     fx_gather<DIM, SH::THREADS, FPB>(m.fst, w, nc, S, f0, nf, ua, ub, ex);
@@ -495,13 +602,23 @@ __global__ void __launch_bounds__(FluxShape<DIM, Q>::THREADS, FluxShape<DIM, Q>:
 #pragma unroll
     for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
     if (live) {
-      if (E != kFxPlain && ex[fi * DIM] != 0) {
-        FxAll<DIM, FPB> a{ua + fi, ub + fi, {}};
-        rw.run(co, S, E, a);
+      bool fx = E != kFxPlain && ex[fi * DIM] != 0;
+      if (fx) {
+        FxAll<DIM, FPB> a{ua + fi, ub + fi, {}, {}};
+        rw.head(co, S, E, a);
+        fx = a.sure(E, ex + fi * DIM);
+        if (fx) {
+          rw.tail(co, HEAD, S, E, a);
 #pragma unroll
-        for (int j = 0; j < DIM; ++j) acc[j] = fx_scale(a.s[j].total(), E, ex[fi * DIM + j]);
-      } else
-        plain_row<DIM>(co, kTile * R, S, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc, acc);
+          for (int j = 0; j < DIM; ++j) acc[j] = fx_scale(a.s[j].total(), E, ex[fi * DIM + j]);
+        }
+      }
+      if (!fx) {
+        const PlainSum<DIM> s =
+            plain_row<DIM, kTile * R>(co, S, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) acc[j] = s.v[j];
+      }
       if (f >= m.nfi && f < m.nfi + m.nfd) {  // ghost node of a displacement face
         const int64_t fd = f - m.nfi;
         const double cg = m.gco[fd * R + r];
