@@ -333,7 +333,7 @@ void launch_row_sums(const DevMesh& m, double* fcsum, cudaStream_t st);
 // coefficient row of a [tiles][S][cs], as the fixed-point contractions scale by
 void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_t* out, cudaStream_t st);
 // raises the dynamic shared-memory limit of the face and extrapolation kernels
-// (once per process, at set-up); 0 or a cudaError_t
+// on the current device (at set-up); 0 or a cudaError_t
 int setup_face_kernels();
 void launch_source(const hofv_ctx* c, cudaStream_t st);
 void launch_build_tco(const DevMesh& m, double mu, double lam, double* tco, cudaStream_t st);

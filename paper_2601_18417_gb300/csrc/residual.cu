@@ -1974,8 +1974,8 @@ void launch_jv_df(const DevMesh& m, const Material& mat, const double* v, const 
 
 // the face kernels' differences and limbs exceed the default 48 KB of dynamic
 // shared memory for large stencils: raise the limit of every instantiation to what
-// kMaxS stencil cells need, once per process (set-up calls only, never
-// during stream capture)
+// kMaxS stencil cells need.  The limit belongs to the device, so each set-up
+// raises it on its own (0.04 ms; never during stream capture)
 template <int DIM, int LAW, int MODE, int QD, bool PACK>
 static void raise_smem(cudaError_t& e) {
   const cudaError_t r =
@@ -2008,8 +2008,6 @@ static void raise_smem_flux(cudaError_t& e) {
   raise_smem_fx(e, k_flux<DIM, HOFV_LAW_NEOHOOKEAN, Q>, FluxShape<DIM, Q>::smem(kMaxS));
 }
 int setup_face_kernels() {
-  static int rc = -1;
-  if (rc >= 0) return rc;
   cudaError_t e = cudaSuccess;
   raise_smem_ustar<2, 3>(e);
   raise_smem_ustar<2, 4>(e);
@@ -2037,8 +2035,7 @@ int setup_face_kernels() {
   raise_smem_all<3, 8>(e);
   raise_smem_all<3, 16>(e);
   raise_smem_all<3, 32, true>(e);
-  rc = e == cudaSuccess ? 0 : (int)e;
-  return rc;
+  return e == cudaSuccess ? 0 : (int)e;
 }
 
 void launch_jv_cache_fill(const DevMesh& m, const Material& mat, const double* u,
