@@ -1297,7 +1297,7 @@ static int arnoldi_launch(hofv_ctx* c, const hofv_solve_opts& o, const ArnoldiKe
   launch_multi_axpy(w, V, dh + k.dstride, nv, n, k.ld, c->stream);
   launch_norm2(w, n, c->d_red, c->d_count, dh + 2 * k.dstride, c->red_blocks, c->stream);
   if (k.with_scale)
-    launch_scale_copy(V + (int64_t)(k.j + 1) * k.ld, w, dh + 2 * k.dstride, 1, n, c->stream);
+    launch_scale_copy(V + (int64_t)(k.j + 1) * k.ld, w, dh + 2 * k.dstride, 1, n, c->red_blocks, c->stream);
   HOFV_CUDA(c, cudaGetLastError());
   return 0;
 }
@@ -1436,7 +1436,7 @@ static int fgmres(hofv_ctx* c, const hofv_solve_opts& o, const double* u, const 
     const bool cycle_gnn = oc.precond == HOFV_PC_GNN;
     bool broken = false;
     HOFV_CUDA(c, cudaMemcpyAsync(c->d_scal + 20, &beta, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    launch_scale_copy(V, r, c->d_scal + 20, 1, n, c->stream);
+    launch_scale_copy(V, r, c->d_scal + 20, 1, n, c->red_blocks, c->stream);
     std::fill(F.g.begin(), F.g.end(), 0.0);
     F.g[0] = beta;
     int j = 0;
@@ -1457,7 +1457,7 @@ static int fgmres(hofv_ctx* c, const hofv_solve_opts& o, const double* u, const 
         launch_dots(V, n, w, j + 1, n, c->d_red, c->d_count, dh + (m + 2), c->red_blocks, c->stream, 0);
         launch_multi_axpy(w, V, dh + (m + 2), j + 1, n, n, c->stream);
         launch_norm2(w, n, c->d_red, c->d_count, dh + 2 * (m + 2), c->red_blocks, c->stream);
-        launch_scale_copy(V + (int64_t)(j + 1) * n, w, dh + 2 * (m + 2), 1, n, c->stream);
+        launch_scale_copy(V + (int64_t)(j + 1) * n, w, dh + 2 * (m + 2), 1, n, c->red_blocks, c->stream);
       } else {
         // v_{j+1} = w / |w| follows at once (with |w| = 0 it is never read)
         const ArnoldiKey key{c->gen, oc.precond, oc.inner_iters, j, 0, 1, u, Ru, V, Z, w, dh,

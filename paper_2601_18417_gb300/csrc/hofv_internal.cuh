@@ -367,7 +367,7 @@ void launch_jv_norms(const double* v, const double* u, int64_t n, double* red, u
 // y = x + sign * alpha[0] * v
 void launch_waxpy_dev(double* y, const double* x, const double* v, const double* alpha,
                       double sign, int64_t n, cudaStream_t st);
-void launch_scale_copy(double* y, const double* x, const double* s, int invert, int64_t n,
+void launch_scale_copy(double* y, const double* x, const double* s, int invert, int64_t n, int blocks,
                        cudaStream_t st);
 void launch_multi_axpy(double* w, const double* V, const double* coef, int k, int64_t n,
                        int64_t ld, cudaStream_t st);

@@ -190,10 +190,10 @@ __global__ void k_scale_copy(double* __restrict__ y, const double* __restrict__ 
        i += (int64_t)gridDim.x * blockDim.x)
     y[i] = x[i] * f;
 }
-void launch_scale_copy(double* y, const double* x, const double* s, int invert, int64_t n,
+void launch_scale_copy(double* y, const double* x, const double* s, int invert, int64_t n, int blocks,
                        cudaStream_t st) {
-  // at most four blocks an SM: 512^2 x 2 7.9 -> 3.6 us with the quotient once a block
-  k_scale_copy<<<(unsigned)std::min<int64_t>((n + 255) / 256, 608), 256, 0, st>>>(y, x, s, invert, n);
+  // four blocks an SM at most: 512^2 x 2 7.9 -> 3.6 us with the quotient once a block
+  k_scale_copy<<<(unsigned)std::min<int64_t>((n + 255) / 256, blocks), 256, 0, st>>>(y, x, s, invert, n);
 }
 
 // w -= sum_k coef[k] V_k  (coef on the device)

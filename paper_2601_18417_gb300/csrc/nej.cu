@@ -285,7 +285,7 @@ int nej_precondition(hofv_ctx* c, int iters, const double* v, double* z) {
   HOFV_CUDA(c, cudaStreamSynchronize(st));
   HOFV_CUDA(c, cudaMemsetAsync(z, 0, sizeof(double) * n, st));
   if (!(beta > 0.0)) return std::isfinite(beta) ? 0 : fail(c, HOFV_ENAN, "non-finite vector");
-  launch_scale_copy(g->V, v, nrm, 1, n, st);
+  launch_scale_copy(g->V, v, nrm, 1, n, c->red_blocks, st);
   std::vector<double> H((size_t)(k + 1) * k, 0.0), cs(k), sn(k), gv(k + 1, 0.0), hb(2 * (k + 2) + 2);
   gv[0] = beta;
   int j = 0;
@@ -306,7 +306,7 @@ int nej_precondition(hofv_ctx* c, int iters, const double* v, double* z) {
     double* Hc = H.data() + (size_t)j * (k + 1);
     for (int i = 0; i <= j; ++i) Hc[i] = hb[i] + hb[(k + 2) + i];
     Hc[j + 1] = hn;
-    if (hn > 0.0 && j + 1 < k) launch_scale_copy(g->V + (int64_t)(j + 1) * n, g->w, nrm + 1, 1, n, st);
+    if (hn > 0.0 && j + 1 < k) launch_scale_copy(g->V + (int64_t)(j + 1) * n, g->w, nrm + 1, 1, n, c->red_blocks, st);
     for (int i = 0; i < j; ++i) {
       const double t = cs[i] * Hc[i] + sn[i] * Hc[i + 1];
       Hc[i + 1] = -sn[i] * Hc[i] + cs[i] * Hc[i + 1];
