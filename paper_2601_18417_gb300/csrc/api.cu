@@ -83,7 +83,6 @@ DevMesh dev_mesh(const hofv_ctx* c) {
   m.vext = c->d_vext;
   m.gcache = c->d_gcache;
   m.tcache = c->d_tcache;
-  m.kerr = c->d_bar ? c->d_bar + 3 : nullptr;
   m.fcsum = c->d_fcsum;
   m.fexp = c->d_fexp;
   m.cexp = c->d_cexp;
@@ -1250,17 +1249,20 @@ struct ArnoldiKey {
   }
 };
 // The projections and the norm of a step (up to 2 * 102 + 1 doubles) and the
-// two error flags come back in one page of pinned memory with one wait.  As four
+// grid barrier's error flag come back in one page of pinned memory with one wait.  As four
 // copies to pageable memory, each waiting by itself, they left the device idle
 // for a quarter of a solve on 12^3 hexes (7.67 -> 5.73 ms with this).
-constexpr int kKryHost = 256;                // doubles; the flags lie in the last one
-static int check_flags(hofv_ctx* c, const int* flags);
+constexpr int kKryHost = 256;                // doubles; the flag lies in the last one
 static int read_step(hofv_ctx* c, const double* dh, int count) {
-  int* flags = reinterpret_cast<int*>(c->h_kry + kKryHost - 1);
+  int* flag = reinterpret_cast<int*>(c->h_kry + kKryHost - 1);
   HOFV_CUDA(c, cudaMemcpyAsync(c->h_kry, dh, sizeof(double) * count, cudaMemcpyDeviceToHost, c->stream));
-  HOFV_CUDA(c, cudaMemcpyAsync(flags, c->d_bar + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  HOFV_CUDA(c, cudaMemcpyAsync(flag, c->d_bar + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   HOFV_CUDA(c, cudaStreamSynchronize(c->stream));
-  return check_flags(c, flags);
+  if (*flag) {
+    HOFV_CUDA(c, cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)));
+    return fail(c, HOFV_ECUDA, "approximate-Jacobian solve: grid barrier timed out");
+  }
+  return 0;
 }
 
 struct GraphCache {
@@ -1830,21 +1832,6 @@ extern "C" int hofv_force_scale(hofv_ctx* c, const double* u, double* fs) {
   if (!std::isfinite(m)) return fail(c, HOFV_ENAN, "non-finite face flux");
   return HOFV_OK;
 }
-
-namespace hofv {
-// the flags as read from d_bar + 2: the grid barrier's, the face kernels'
-static int check_flags(hofv_ctx* c, const int* flags) {
-  if (flags[0]) {
-    HOFV_CUDA(c, cudaMemset(c->d_bar, 0, 4 * sizeof(unsigned int)));
-    return fail(c, HOFV_ECUDA, "approximate-Jacobian solve: grid barrier timed out");
-  }
-  if (flags[1]) {
-    HOFV_CUDA(c, cudaMemset(c->d_bar + 3, 0, sizeof(unsigned int)));
-    return fail(c, HOFV_ECUDA, "face kernel: a shared-memory copy did not complete in time");
-  }
-  return 0;
-}
-}  // namespace hofv
 
 extern "C" int hofv_selftest_barrier(hofv_ctx* c, int32_t* timed_out) {
   if (!c || !timed_out) return HOFV_EINVAL;

@@ -95,7 +95,6 @@ struct DevMesh {
   // (by plane, as the pairs)
   double* gcache;         // [nftile][dim][dim][kTile * Q]
   double* tcache;         // [nftile][dim][kTile * Q]
-  unsigned int* kerr;     // set to 1 by a face kernel whose bounded wait ran out
   const uint16_t* fexp;   // [nftile][kTile][R] largest biased exponent of each gradient row
   const uint16_t* cexp;   // [nctile][kTile][nlf] ... of each extrapolation row (HOFV_PREC_FP64)
   const double* fcsum;    // [nftile][dim][kTile * Q] sums over the stencil of the stored
@@ -212,7 +211,8 @@ struct hofv_ctx {
   double* d_aj_off = nullptr;       // [nc][nlf]
   float* d_aj_diag32 = nullptr;
   float* d_aj_off32 = nullptr;
-  unsigned int* d_bar = nullptr;    // grid barrier of the persistent CG: arrivals, blocks done, error
+  unsigned int* d_bar = nullptr;    // grid barrier of the persistent CG: arrivals, blocks done, error,
+                                    // and a word of its self-test
   double* d_aj_invd = nullptr;      // 1 / (-diag), FP64 and FP32
   float* d_aj_invd32 = nullptr;
   // CG work vectors

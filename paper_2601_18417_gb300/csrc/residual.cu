@@ -1190,18 +1190,6 @@ __device__ __forceinline__ float2 ld_pair(const float2* __restrict__ pl, int i, 
   return (i & 1) ? make_float2(h.y, l.y) : make_float2(h.x, l.x);
 }
 
-// split state of cell `id` as double-float pairs (hi, mid): 48 bits
-template <int DIM>
-__device__ __forceinline__ void ld_split(const float4* __restrict__ p, int32_t id, float (&h)[DIM],
-                                         float (&l)[DIM]) {
-#pragma unroll
-  for (int j = 0; j < DIM; ++j) {
-    const float4 a = __ldg(p + (int64_t)id * DIM + j);
-    h[j] = a.x;
-    l[j] = a.y;
-  }
-}
-
 __device__ __forceinline__ void split_value(double a, float& h, float& l) {
   h = __double2float_rn(a);
   l = __double2float_rn(a - (double)h);  // a - h is exact in FP64
