@@ -317,7 +317,7 @@ struct UstarShape {
   static constexpr int CPB = DIM == 2 ? 32 : 16;
   static constexpr int ROWS = CPB * NLF;
   // four threads a row: 32^3 hexes 73 -> 59 us; two on 512^2 quads 57 -> 71 (both
-  // before the sums were checked, 70 and 67 now)
+  // before the sums were checked, 70 and 67 now); 6 17^3 tetrahedra 64 -> 42
   static constexpr int W = NLF >= 8 || DIM == 2 ? 1 : 4;
   static constexpr int THREADS = ROWS * W;
   static constexpr int BLOCKS = 1152 / THREADS;
@@ -1455,9 +1455,13 @@ __device__ __forceinline__ double mirror_i(const double* x, const double* n, int
 // a Jacobian-vector product: one thread a coefficient row before -> this):
 // 48^3 hexes p = 3 neo-Hookean 1554 -> 1132, 48^3 hexes p = 2 807 -> 502,
 // 512^2 quads p = 3 linear 197 -> 129, 24-layer prisms 524 -> 344, 6 17^3
-// tetrahedra 158 -> 104.  The coefficient stream is 85 % of measured HBM at
-// p = 3; the rest is the FP64 law (without it: 1009 of 1266 us at that stage)
-// and, at p = 2, the gather of the differences (442 of 582 us without).
+// tetrahedra 158 -> 104; 32^3 hexes face by face (16 points a face) 670 -> 453,
+// neo-Hookean 846 -> 502, with one point a fan slot (4) 178 -> 121, 24-layer
+// prisms with one (8) 207 -> 129, 200^2 polygons (2) 57 -> 35.  The coefficient
+// stream is 85 % of measured HBM at p = 3; the rest is the FP64 law (without it:
+// 1009 of 1266 us at that stage) and, at p = 2, the gather of the differences (442
+// of 582 us without).  A plane of a prism's triangle is 96 bytes, which DRAM
+// reads as 128: 11 % more bytes than needed on prisms (4 % with a face's rows together).
 //  * A thread a point instead of a row: a difference read from shared memory
 //    serves DIM rows, the gradient never leaves registers, and no barrier
 //    stands between contraction and law, so one warp's FP64 law runs beside
