@@ -14,6 +14,7 @@ import numpy as np
 import pytest
 
 from tests import helpers as H
+from tests.test_gpu_polyhedra import _context as polyhedral_context
 
 pytestmark = pytest.mark.gpu
 LD = np.longdouble
@@ -59,7 +60,8 @@ def _reference(ctx, pb, u, absolute):
 def test_terms_of_very_different_size(dim, n, p, q1, kind):
     import torch
     pb = H.make_problem(dim, n, p, q1, jitter=0.15, seed=3, kind=kind, alpha=ALPHA)
-    ctx = H.gpu_context(pb)
+    # boundary data at the library's points, which may be more than the oracle's
+    ctx = polyhedral_context(pb) if kind == "polyhedron" else H.gpu_context(pb)
     g, nc = np.random.default_rng(7), pb.orc.nc
     states = []
     for cell in (nc // 2, int(g.integers(nc))):
