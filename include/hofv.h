@@ -298,7 +298,7 @@ int hofv_set_contraction(hofv_ctx* ctx, int on);
    gradient at every face Gauss point, eq. faceQuadGrad, and the
    extrapolated face values of the stabilisation, eq. alphaJump).
    HOFV_PREC_FP64 (default) takes FP64 coefficients and values.  Where a row's
-   first products are large enough against its largest coefficient times the
+   products are large enough against its largest coefficient times the
    stencil's largest value, their sum is formed in 64-bit fixed point and
    rounded once, which leaves a smaller error than FP64 fused multiply-adds
    (a tenth on smooth fields); elsewhere (values that differ by orders of

@@ -18,9 +18,9 @@ namespace hofv {
 constexpr int kFxMin = 555, kFxMax = 1560;  // biased exponents: the scales stay normal numbers
 constexpr int kFxZero = kFxMin - 1;         // exponent of a row or a stencil of zeros
 constexpr uint16_t kFxPlain = 0xffff;       // row exponent of a row to be summed by FMAs
-// A sum is taken as exact enough where its first products (the nearest cells',
-// whose coefficients are the largest) add up to this in magnitude, in units of
-// 2^32 of the high limbs' products: 2^55 of those in 2-D, 2^54 in 3-D, where four
+// A sum is taken as exact enough where some of its products, the nearest cells'
+// with the largest coefficients among them, add up to this in magnitude, in units
+// of 2^32 of the high limbs' products: 2^55 of those in 2-D, 2^54 in 3-D, where four
 // times the slots make FMAs err more (residual.cu has the figures).
 HOFV_HD constexpr uint32_t fx_sure(int dim) { return dim == 2 ? 1u << 23 : 1u << 22; }
 

@@ -51,30 +51,33 @@ namespace hofv {
 // the error of FMAs with the partial sums.  Where the products are all small
 // against those maxima (one value among zeros, a far cell's large value, a
 // field falling by ten a cell) FMAs are the more accurate, and they are taken
-// then: a row's sum is left in fixed point only if its first products add up to
-// 2^-4 (2-D) or 2^-5 (3-D) of 2^e times the values' binade (fx_sure).
+// then: a row's sum is left in fixed point only if some of its products, the nearest
+// cells' among them, add up to 2^-4 (2-D) or 2^-5 (3-D) of 2^e times the values'
+// binade (fx_sure, fx_row).
 // Errors of this rule and of FMAs alone over sum |c_N u_N|, rms over the gradient
 // rows of jittered p = 3 hexes (quads), and the rows left in fixed point:
 //   smooth field         1.7e-17 and 1.5e-16 (1.3e-17 and 5.6e-17)   all
 //   random values        1.8e-17 and 1.3e-16 (3.4e-17 and 1.1e-16)   all (99 %)
-//   zero across the face 2.0e-17 and 1.6e-16 (3.2e-17 and 1.2e-16)   99.9 % (98.9 %)
+//   zero across the face 2.0e-17 and 1.6e-16 (3.2e-17 and 1.2e-16)   all (98.9 %)
 //   falling by e a cell  4.2e-17 and 9.2e-17 (4.1e-17 and 6.1e-17)   99.9 % (85 %)
-//   falling by 10 a cell 8.7e-17 and 1.0e-16 (5.7e-17 and 6.5e-17)   19 % (8 %)
-//   one value            4.6e-17 and 4.6e-17 (4.7e-17 and 4.7e-17)   12 % (9 %)
+//   falling by 10 a cell 9.2e-17 and 1.0e-16 (5.7e-17 and 6.5e-17)   28 % (8 %)
+//   one value            4.6e-17 and 4.6e-17 (4.7e-17 and 4.7e-17)   6 % (9 %)
 //
 // What bounds it: integer issue.  A coefficient takes about 17 instructions to
 // split and, for three components, nine multiply-adds at 32 a clock and SM (209
-// of the 499 us on 32^3 hexes; the bytes take 257).  Measured on smooth fields,
-// FP64 FMAs alone -> this (us): k_flux 32^3 hexes p = 3 neo-Hookean 1427 -> 499,
-// 40^3 p = 2 1077 -> 380, 2 255^2 triangles 110 -> 78, 20-layer prisms 1104 -> 420,
-// 6 17^3 tetrahedra 272 -> 136; k_ustar 32^3 hexes 107 -> 70, 40^3 148 -> 101, 512^2
-// quads 83 -> 67.  Without the check and the way to FMAs the same rows took 476,
-// 355, 76, 390, 119, 65, 97 and 65, the tetrahedra among them because 0.1 % of their
-// rows go that way.  A state that takes nearly all rows there (values spread
-// over 2^40): k_flux 1322, 934, 137, 981, 293, k_ustar 119, 175, 107.  Strides known to the
-// compiler and a loop without range checks gave 666 -> 497 of the first.  Not
-// kept: every 5th slot by FP64 FMAs beside the others (515 for 467), two of five
-// (682); the FMAs behind a barrier (516 for 499) or inlined (504); the limbs cut from
+// of the 494 us on 32^3 hexes; the bytes take 257).  Measured on smooth fields,
+// FP64 FMAs alone -> this (without the check and the way to FMAs), us: k_flux 32^3
+// hexes p = 3 neo-Hookean 1427 -> 494 (475), 12^3 45 (41), 20^3 151 (132: one row's
+// FMAs), 40^3 p = 2 1077 -> 385 (355), 2 255^2 triangles 110 -> 81 (76), 20-layer
+// prisms 1104 -> 426 (390), 6 17^3 tetrahedra 272 -> 132 (119); k_ustar 32^3 hexes
+// 107 -> 73 (65), 40^3 148 -> 106 (97), 512^2 quads 83 -> 68 (65).  A state that takes
+// nearly all rows to FMAs (values spread over 2^40): k_flux 1326, 937, 134, 982, 298
+// (32^3, 40^3, triangles, prisms, tetrahedra), k_ustar 122, 178, 103.  Strides known to
+// the compiler and a loop without range checks gave 666 -> 497 of the first when
+// nothing was checked.  Not kept: every 5th slot by FP64 FMAs beside the others (515
+// for 467), two of five (682); the FMAs behind a barrier (516 for 499) or inlined (504);
+// a lone row's FMAs with a lane a slot, or its operands loaded ahead (no gain); the
+// second look out of line (a state spread over 2^40: 2053 for 1326); the limbs cut from
 // one 64-bit integer (684).
 //
 // Rows and stencils whose largest binade lies outside [kFxMin, kFxMax] (tiny,
@@ -182,36 +185,40 @@ __device__ __forceinline__ void fx_gather(const int32_t* __restrict__ sten, cons
   __syncthreads();
 }
 
-// Streams the S coefficients of the row co (CS between slots) as limbs, the
-// first HEAD to mac.head(limbs, n), those from n0 on to mac(limbs, n0, d),
-// slot n0 + d; E is the row's exponent.  K slots are requested ahead in registers
-// (begin, before the values are ready).
-template <int K, int CS, int HEAD>
+// Streams the S coefficients of the row co (CS between slots) as limbs to
+// mac(limbs, n0, d), slot n0 + d, or, with CHECK, to mac.check(limbs, n); E is the
+// row's exponent.  K slots are requested ahead in registers (begin, before the
+// values are ready); K slots from n0 (round), all from n0 on (rest).
+template <int K, int CS>
 struct FxRow {
-  static_assert(HEAD % K == 0, "the head takes whole rounds of requests");
   double c[K];
   __device__ __forceinline__ void begin(const double* __restrict__ co, int S) {
 #pragma unroll
     for (int d = 0; d < K; ++d) c[d] = d < S ? __ldg(co + d * CS) : 0.0;
   }
-  template <typename F>
-  __device__ __forceinline__ void head(const double* __restrict__ co, int S, int E, F& mac) {
-#pragma unroll
-    for (int n = 0; n < HEAD; ++n) {
-      const FxLimbs q = fx_coef(c[n % K], E);
-      if (n + K < S) c[n % K] = __ldg(co + (n + K) * CS);
-      if (n < S) mac.head(q, n);
-    }
+  template <bool CHECK, typename F>
+  static __device__ __forceinline__ void put(FxLimbs q, int n0, int d, F& mac) {
+    if constexpr (CHECK) mac.check(q, n0 + d);
+    else mac(q, n0, d);
   }
   template <typename F>
-  __device__ __forceinline__ void tail(const double* __restrict__ co, int n0, int S, int E, F& mac) {
+  __device__ __forceinline__ void round(const double* __restrict__ co, int n0, int S, int E, F& mac) {
+#pragma unroll
+    for (int d = 0; d < K; ++d) {
+      const FxLimbs q = fx_coef(c[d], E);
+      if (n0 + K + d < S) c[d] = __ldg(co + (n0 + K + d) * CS);
+      if (n0 + d < S) mac.check(q, n0 + d);
+    }
+  }
+  template <bool CHECK, typename F>
+  __device__ __forceinline__ void rest(const double* __restrict__ co, int n0, int S, int E, F& mac) {
     co += (n0 + K) * CS;
     for (; n0 + 2 * K <= S; n0 += K) {  // every request in range
 #pragma unroll
       for (int d = 0; d < K; ++d) {
         const FxLimbs q = fx_coef(c[d], E);
         c[d] = __ldg(co + d * CS);
-        mac(q, n0, d);
+        put<CHECK>(q, n0, d, mac);
       }
       co += K * CS;
     }
@@ -219,11 +226,11 @@ struct FxRow {
     for (int d = 0; d < K; ++d) {
       const FxLimbs q = fx_coef(c[d], E);
       if (n0 + K + d < S) c[d] = __ldg(co + d * CS);
-      if (n0 + d < S) mac(q, n0, d);
+      if (n0 + d < S) put<CHECK>(q, n0, d, mac);
     }
 #pragma unroll
     for (int d = 0; d < K; ++d)
-      if (n0 + K + d < S) mac(fx_coef(c[d], E), n0, K + d);
+      if (n0 + K + d < S) put<CHECK>(fx_coef(c[d], E), n0, K + d, mac);
   }
 };
 
@@ -243,7 +250,7 @@ struct FxAll {
       s[2].mac(q, b.x, b.y);
     }
   }
-  __device__ __forceinline__ void head(FxLimbs q, int n) {
+  __device__ __forceinline__ void check(FxLimbs q, int n) {
     (*this)(q, n, 0);
     const int4 a = ua[n * STRIDE];
     size[0] += fx_size(q, a.x);
@@ -251,14 +258,49 @@ struct FxAll {
     if constexpr (DIM == 3) size[2] += fx_size(q, ub[n * STRIDE].x);
   }
   // the sums are exact enough, or all coefficients (exponent E) or values
-  // (exponents ex) are zero
-  __device__ __forceinline__ bool sure(int E, const int* ex) const {
+  // (exponents ex) are zero; least: the size that is enough
+  __device__ __forceinline__ bool sure(int E, const int* ex, uint32_t least = fx_sure(DIM)) const {
     bool r = true;
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) r &= size[j] >= fx_sure(DIM) || ex[j] == kFxZero;
+    for (int j = 0; j < DIM; ++j) r &= size[j] >= least || ex[j] == kFxZero;
     return r || E == kFxZero;
   }
+  // sure from here on: a size stays below 15 2^26 by the scale of the row
+  __device__ __forceinline__ void pass() {
+#pragma unroll
+    for (int j = 0; j < DIM; ++j) size[j] += 1u << 30;
+  }
 };
+
+// All slots of a row whose exponents are in range (fx); true if the sum stands.
+// Ten slots are checked, the nearest cells.  In 3-D a row that does not pass by them,
+// but comes within a factor 4 (noise: 1e-5 to 1e-3 of the rows of smooth fields),
+// is judged by all its slots, with 5/4 as the bar, since what is left out weighs
+// more where the far cells' values decide; its warp then checks them all.  A lone
+// row's FMAs would hold its block up by 20 us (a chain of 85 slots, 2400 cycles for
+// four).  The rule looks at a row's own values only, so that a face's flux depends
+// on its stencil alone to the last bit.  Called by whole warps in 3-D.
+template <int K, int CS, int DIM, int STRIDE>
+__device__ __forceinline__ bool fx_row(FxRow<K, CS>& r, const double* __restrict__ co, int S, int E, const int* ex,
+                                       bool fx, FxAll<DIM, STRIDE>& a) {
+  bool ok = false, near = false;
+  if (fx) {
+    r.round(co, 0, S, E, a);
+    r.round(co, K, S, E, a);
+    ok = a.sure(E, ex);
+    near = DIM == 3 && a.sure(E, ex, fx_sure(DIM) / 4);
+  }
+  if (DIM == 3 && __any_sync(0xffffffffu, near && !ok)) {
+    if (near) {
+      if (ok) a.pass();
+      r.template rest<true>(co, 2 * K, S, E, a);
+      ok = a.sure(E, ex, fx_sure(DIM) / 4 * 5);
+    }
+  } else if (ok) {
+    r.template rest<false>(co, 2 * K, S, E, a);
+  }
+  return ok;
+}
 
 // the same sum by FP64 FMAs, SL slots CS apart, U slots' requests at a time
 template <int DIM>
@@ -317,7 +359,7 @@ struct UstarShape {
   static constexpr int CPB = DIM == 2 ? 32 : 16;
   static constexpr int ROWS = CPB * NLF;
   // four threads a row: 32^3 hexes 73 -> 59 us; two on 512^2 quads 57 -> 71 (both
-  // before the sums were checked, 70 and 67 now); 6 17^3 tetrahedra 64 -> 42
+  // before the sums were checked, 73 and 68 now); 6 17^3 tetrahedra 64 -> 44
   static constexpr int W = NLF >= 8 || DIM == 2 ? 1 : 4;
   static constexpr int THREADS = ROWS * W;
   static constexpr int BLOCKS = 1152 / THREADS;
@@ -334,7 +376,7 @@ __global__ void __launch_bounds__(UstarShape<DIM, NLF>::THREADS, UstarShape<DIM,
   constexpr int CPB = SH::CPB, ROWS = SH::ROWS, W = SH::W, CS = kTile * NLF;
   extern __shared__ __align__(16) double sm[];
   __shared__ int ex[CPB * DIM];
-  __shared__ uint8_t sure[W > 1 ? ROWS : 1];  // FxAll::sure of the row's first part
+  __shared__ uint32_t size[W > 1 ? W * DIM * ROWS : 1];  // the parts' FxAll::size
   const int S = m.S;
   int4* ua = reinterpret_cast<int4*>(sm);                                        // [S][CPB]
   int2* ub = reinterpret_cast<int2*>(ua + S * CPB);                              // [S][CPB]
@@ -348,37 +390,42 @@ __global__ void __launch_bounds__(UstarShape<DIM, NLF>::THREADS, UstarShape<DIM,
   const int row = (int)(cell % kTile) * NLF + lf;
   const int n0 = p * S / W, len = (p + 1) * S / W - n0;  // this thread's slots
   const double* __restrict__ co = m.cex + tile * (int64_t)S * CS + row + (int64_t)n0 * CS;
-  constexpr int HEAD = 10;
-  FxRow<5, CS, HEAD> r;
+  FxRow<5, CS> r;
   r.begin(co, on ? len : 0);
   const int E = on ? m.cexp[tile * CS + row] : kFxPlain;
   const int64_t ws = m.wst;  // stride of the state read
   fx_gather<DIM, SH::THREADS, CPB>(m.cst, w, ws, S, cell0, (int)min((int64_t)CPB, m.nc - cell0), ua, ub, ex);
   bool fx = E != kFxPlain && ex[ci * DIM] != 0;
   FxTotal t[DIM];
-  if (fx) {
-    FxAll<DIM, CPB> a{ua + n0 * CPB + ci, ub + n0 * CPB + ci, {}, {}};
-    if (p == 0) {
-      r.head(co, len, E, a);
-      const bool ok = a.sure(E, ex + ci * DIM);
-      if (W == 1) fx = ok;
-      else sure[it] = ok;
-    }
-    if (fx) r.tail(co, p == 0 ? HEAD : 0, len, E, a);
+  FxAll<DIM, CPB> a{ua + n0 * CPB + ci, ub + n0 * CPB + ci, {}, {}};
+  if (W == 1) {
+    if (DIM == 3 || fx) fx = fx_row(r, co, len, E, ex + ci * DIM, fx, a);
+  } else if (fx) {  // ten slots of the first part are checked, five of each other
+    r.round(co, 0, len, E, a);
+    if (p == 0) r.round(co, 5, len, E, a);
+    r.template rest<false>(co, p == 0 ? 10 : 5, len, E, a);
 #pragma unroll
-    for (int j = 0; j < DIM; ++j) t[j] = a.s[j].total();
+    for (int j = 0; j < DIM; ++j) size[(p * DIM + j) * ROWS + it] = a.size[j];
+  }
+#pragma unroll
+  for (int j = 0; j < DIM; ++j) {
+    t[j] = a.s[j].total();
     if (W > 1 && p > 0) {
-#pragma unroll
-      for (int j = 0; j < DIM; ++j) {
-        part[((p - 1) * DIM + j) * ROWS + it] = t[j].h;
-        part_l[((p - 1) * DIM + j) * ROWS + it] = t[j].l;
-      }
+      part[((p - 1) * DIM + j) * ROWS + it] = t[j].h;
+      part_l[((p - 1) * DIM + j) * ROWS + it] = t[j].l;
     }
   }
-  bool again = !fx;  // some row of the block is to be summed by FMAs
+  bool again = W == 1 && !fx;  // some row of the block is to be summed by FMAs
   if (W > 1) {
     __syncthreads();
-    fx = fx && sure[it];
+    if (fx) {
+#pragma unroll
+      for (int j = 0; j < DIM; ++j)
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          if (k != p) a.size[j] += size[(k * DIM + j) * ROWS + it];
+      fx = a.sure(E, ex + ci * DIM);
+    }
     again = __syncthreads_or(on && !fx);
   }
   PlainSum<DIM> acc;
@@ -591,34 +638,28 @@ __global__ void __launch_bounds__(FluxShape<DIM, Q>::THREADS, FluxShape<DIM, Q>:
     // corner) are neither read nor formed
     const bool live = fi < nf && (m.fql == nullptr || r < __ldg(m.fql + f) * DIM);
     const double* __restrict__ co = m.fco + tile * (int64_t)S * kTile * R + row;
-    // slots that are checked: the nearest ring of cells (with 10 on tetrahedra one
-    // warp in twelve went on to FMAs)
-    constexpr int HEAD = DIM == 2 ? 10 : 15;
-    FxRow<5, kTile * R, HEAD> rw;
+    FxRow<5, kTile * R> rw;
     rw.begin(co, live ? S : 0);
     const int E = live ? m.fexp[tile * kTile * R + row] : kFxPlain;
     fx_gather<DIM, SH::THREADS, FPB>(m.fst, w, nc, S, f0, nf, ua, ub, ex);
     double acc[DIM];
 #pragma unroll
     for (int j = 0; j < DIM; ++j) acc[j] = 0.0;
-    if (live) {
-      bool fx = E != kFxPlain && ex[fi * DIM] != 0;
+    if (DIM == 3 || live) {
+      FxAll<DIM, FPB> a{ua + fi, ub + fi, {}, {}};
+      const bool fx = fx_row(rw, co, S, E, ex + fi * DIM, live && E != kFxPlain && ex[fi * DIM] != 0, a);
       if (fx) {
-        FxAll<DIM, FPB> a{ua + fi, ub + fi, {}, {}};
-        rw.head(co, S, E, a);
-        fx = a.sure(E, ex + fi * DIM);
-        if (fx) {
-          rw.tail(co, HEAD, S, E, a);
 #pragma unroll
-          for (int j = 0; j < DIM; ++j) acc[j] = fx_scale(a.s[j].total(), E, ex[fi * DIM + j]);
-        }
+        for (int j = 0; j < DIM; ++j) acc[j] = fx_scale(a.s[j].total(), E, ex[fi * DIM + j]);
       }
-      if (!fx) {
+      if (live && !fx) {
         const PlainSum<DIM> s =
             plain_row<DIM, kTile * R>(co, S, m.fst + tile * (int64_t)S * kTile + f % kTile, w, nc);
 #pragma unroll
         for (int j = 0; j < DIM; ++j) acc[j] = s.v[j];
       }
+    }
+    if (live) {
       if (f >= m.nfi && f < m.nfi + m.nfd) {  // ghost node of a displacement face
         const int64_t fd = f - m.nfi;
         const double cg = m.gco[fd * R + r];
