@@ -55,7 +55,8 @@ def _reference(ctx, pb, u, absolute):
 
 @pytest.mark.parametrize("dim,n,p,q1,kind", [(2, 12, 2, 2, "tensor"), (2, 11, 3, 3, "tensor"),
                                              (2, 8, 3, 2, "simplex"), (3, 6, 2, 2, "tensor"),
-                                             (3, 6, 3, 3, "tensor"), (3, 4, 2, 2, "simplex"),
+                                             (3, 6, 3, 3, "tensor"), (3, 5, 1, 1, "tensor"),
+                                             (3, 4, 1, 1, "simplex"), (3, 4, 2, 2, "simplex"),
                                              (3, 5, 2, 2, "polyhedron")])
 def test_terms_of_very_different_size(dim, n, p, q1, kind):
     import torch
