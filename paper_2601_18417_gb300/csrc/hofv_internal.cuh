@@ -95,7 +95,7 @@ struct DevMesh {
   // (by plane, as the pairs)
   double* gcache;         // [nftile][dim][dim][kTile * Q]
   double* tcache;         // [nftile][dim][kTile * Q]
-  const uint16_t* fexp;   // [nftile][kTile][R] largest biased exponent of each gradient row
+  const uint16_t* fexp;   // [nftile][kTile][R] exponent that scales each gradient row (fx_row_exponent)
   const uint16_t* cexp;   // [nctile][kTile][nlf] ... of each extrapolation row (HOFV_PREC_FP64)
   const double* fcsum;    // [nftile][dim][kTile * Q] sums over the stencil of the stored
                           // (double-float) gradient coefficients of each row
@@ -187,7 +187,7 @@ struct hofv_ctx {
   float4* d_sv = nullptr;           // [nc + ng][split4] split Jv direction
   double* d_ustar_v = nullptr;      // [nc][nlf][dim]
   double* d_fcsum = nullptr;        // [nftile][dim][kTile * Q] row sums of the stored coefficients
-  uint16_t* d_fexp = nullptr;       // [nftile][kTile][R], FP64: row exponents of fco
+  uint16_t* d_fexp = nullptr;       // [nftile][kTile][R], FP64: scale exponents of fco's rows
   uint16_t* d_cexp = nullptr;       // [nctile][kTile][nlf] ... of cex
   double* d_vext = nullptr;         // [dim][nc + ng]
   // neo-Hookean double-float Jv: face gradients and tractions at u, valid
@@ -329,8 +329,8 @@ void launch_coef_format(double* a, int64_t chunks, int np, int rows, int to_df, 
 // fcsum = sum over the stencil slots of the stored coefficients
 // (double-float pairs summed in FP64, in slot order)
 void launch_row_sums(const DevMesh& m, double* fcsum, cudaStream_t st);
-// out[tile][row] = the largest biased exponent over the S slots of each
-// coefficient row of a [tiles][S][cs], as the fixed-point contractions scale by
+// out[tile][row] = the exponent by which the fixed-point contractions scale
+// each coefficient row of a [tiles][S][cs] (fx_row_exponent)
 void launch_row_exponents(const double* a, int S, int cs, int64_t tiles, uint16_t* out, cudaStream_t st);
 // raises the dynamic shared-memory limit of the face and extrapolation kernels
 // on the current device (at set-up); 0 or a cudaError_t
